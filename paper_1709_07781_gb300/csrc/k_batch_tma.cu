@@ -160,8 +160,7 @@ __global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_batch_tma(const BatchA
             pl.pred.kind = int32_t(w(12));
             pl.pred.a = w(13);
             pl.pred.b = w(14);
-            pl.pred.c = w(15);
-            pl.pred.d = w(16);
+            pl.pred.s = w(15);
             pl.mul = w(17);
             pl.n = w(18);
             pl.tiles = w(19);

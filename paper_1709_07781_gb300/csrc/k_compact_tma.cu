@@ -10,10 +10,10 @@ using namespace tma;
 
 namespace {
 
-// tile (768, 16): 26 compute warps, 13312 entries, 4 stages of 52 KiB and a 13 KiB
-//                 spill ring (8 slots of 16 entries per warp), 1 block per SM;
-// tile (512, 16): 16 compute warps, 8192 entries, 3 stages of 32 KiB, 2 blocks per SM;
-// tile (256, 16): 8 compute warps, 4096 entries, 4 stages of 16 KiB, 3 blocks per SM.
+// Compaction, tile (768, 16): 22 compute warps, 11264 entries, 5 tiles of 44 KiB, 1 block per SM;
+//             tile (512, 16): 16 compute warps, 8192 entries, 3 tiles of 32 KiB, 2 blocks per SM;
+//             tile (256, 16): 8 compute warps, 4096 entries, 4 tiles of 16 KiB, 3 blocks per SM.
+// Scan: the same, except 26 compute warps and 4 stages of 52 KiB for (768, 16).
 ka_status launch_tma(const TmaArgs &a, ka_tile tile, bool scan, int32_t pk, uint64_t cap, cudaStream_t stream) {
     if (tile.block == 768) return launch_tma_768(a, scan, pk, cap, stream);
     if (tile.block == 512) return launch_tma_512(a, scan, pk, cap, stream);
@@ -32,7 +32,7 @@ bool compact_tma_eligible(const CompactLaunch &L) {
 }
 
 ka_status launch_compact_tma(const CompactLaunch &L, cudaStream_t stream) {
-    TmaArgs a;
+    TmaArgs a{};
     a.lead = uint32_t(reinterpret_cast<uintptr_t>(L.in) & 15u) / 4u;
     a.in = L.in - a.lead;
     a.out = L.out;
@@ -48,9 +48,38 @@ ka_status launch_compact_tma(const CompactLaunch &L, cudaStream_t stream) {
     return launch_tma(a, L.tile, false, L.pred.kind, L.n + a.lead, stream);
 }
 
+ka_status launch_compact_chain(const ChainLaunch &L, cudaStream_t stream) {
+    const uint64_t entries = L.in2 ? 2 * L.n : L.n;
+    if (entries > kChainEntries || L.chain.n == 0 || L.chain.n > kChainMax) return KA_E_ARG;
+    if (L.n && (!L.in || !L.out)) return KA_E_ARG;
+    if (!L.count || L.n_ptr == L.count) return KA_E_ARG;
+    if (L.in2 && ((reinterpret_cast<uintptr_t>(L.in) | reinterpret_cast<uintptr_t>(L.in2)) & 15u)) return KA_E_ARG;
+    // the compaction's shape when it is one of the two that have chain
+    // kernels, else the smaller of those
+    ka_tile t = resolve_tile(KA_KERNEL_COMPACT, entries, nullptr);
+    if (t.block != 768) t = ka_tile{512, 16};
+    const ka_status ws_ok = check_workspace(L.ws, L.ws_bytes, tiles_for(entries, t.block * t.ipt));
+    if (ws_ok != KA_OK) return ws_ok;
+    TmaArgs a{};
+    a.lead = uint32_t(reinterpret_cast<uintptr_t>(L.in) & 15u) / 4u;
+    a.in = L.in - a.lead;
+    a.in2 = L.in2;
+    a.out = L.out;
+    a.n_ptr = L.n_ptr;
+    a.count = L.count;
+    a.ws = static_cast<WsHeader *>(L.ws);
+    a.status = reinterpret_cast<uint64_t *>(static_cast<char *>(L.ws) + kWsHeaderBytes);
+    a.n = uint32_t(L.n);
+    a.status_cap = status_capacity(L.ws_bytes);
+    a.mul = L.chain.mul_all;
+    a.chain = L.chain;
+    return t.block == 768 ? launch_chain_768(a, entries + a.lead, stream)
+                          : launch_chain_512(a, entries + a.lead, stream);
+}
+
 ka_status launch_scan_tma(const uint32_t *in, uint64_t n, const uint32_t *n_ptr, uint32_t *out, uint32_t *total,
                           void *ws, uint64_t ws_bytes, ka_tile tile, cudaStream_t stream) {
-    TmaArgs a;
+    TmaArgs a{};
     a.lead = uint32_t(reinterpret_cast<uintptr_t>(in) & 15u) / 4u;
     a.in = in - a.lead;
     a.out = out;

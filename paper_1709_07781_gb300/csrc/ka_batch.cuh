@@ -10,6 +10,7 @@ namespace ka {
 
 struct ItemPlan {  // 32 bytes
     PredDev pred;
+    uint32_t spare;
     uint32_t mul;
     uint32_t n;
     uint32_t tiles;

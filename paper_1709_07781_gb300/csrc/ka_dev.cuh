@@ -95,11 +95,15 @@ __device__ __forceinline__ void record_error(WsHeader *ws, uint32_t code, uint32
 //   kAndMaskEq0: keep (x & a) == 0
 //   kLt:         keep x < a            (also (x >> 28) < p, as x < p << 28)
 //   kPopcOdd:    keep popcount(x) odd
-//   kModNe0:     keep x % d != 0, d = 2^c * d' (d' odd), tested without a
-//                division: x is a multiple of d iff its low c bits are zero and
-//                (x >> c) * inverse(d') mod 2^32 <= floor((2^32 - 1) / d')
+//   kModNe0:     keep x % d != 0, d = 2^s * d' (d' odd), tested without a
+//                division: x is a multiple of d iff x * inverse(d') mod 2^32,
+//                rotated right by s, is at most floor((2^32 - 1) / d)
 //                (Granlund & Montgomery 1994, divisibility by an invariant
-//                integer). a = inverse(d'), b = that bound, c = low-bit mask.
+//                integer: for a multiple the product is x / d', whose low s
+//                bits are zero exactly for a multiple of d, and the rotation
+//                puts any other low bits above the bound). a = inverse(d'),
+//                b = that bound, s = shift. One multiply, one rotation and one
+//                comparison an entry.
 //   kNe:         keep x != a
 //   kAll:        keep everything
 // ---------------------------------------------------------------------------
@@ -107,7 +111,7 @@ enum PredKind : int32_t { kAndMaskEq0 = 0, kLt = 1, kPopcOdd = 3, kModNe0 = 4, k
 
 struct PredDev {
     int32_t kind;
-    uint32_t a, b, c, d;  // see the table above; d = shift c of kModNe0
+    uint32_t a, b, s;  // see the table above
 };
 
 __host__ __device__ __forceinline__ uint32_t popc32(uint32_t x) {
@@ -115,6 +119,15 @@ __host__ __device__ __forceinline__ uint32_t popc32(uint32_t x) {
     return __popc(x);
 #else
     return (uint32_t)__builtin_popcount(x);
+#endif
+}
+
+// x rotated right by s < 32 places.
+__host__ __device__ __forceinline__ uint32_t rotr32(uint32_t x, uint32_t s) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_r(x, x, s);
+#else
+    return (x >> s) | (x << ((32u - s) & 31u));
 #endif
 }
 
@@ -153,9 +166,8 @@ __host__ __device__ __forceinline__ int pred_canon(int32_t kind, uint32_t param,
         }
         p.kind = kModNe0;
         p.a = inverse_odd(odd);
-        p.b = 0xFFFFFFFFu / odd;
-        p.c = shift == 0 ? 0u : (0xFFFFFFFFu >> (32 - shift));
-        p.d = shift;
+        p.b = 0xFFFFFFFFu / param;
+        p.s = shift;
         break;
     }
     case 5: p.kind = kNe; p.a = param; break;          // KA_PRED_NE
@@ -171,7 +183,7 @@ __host__ __device__ __forceinline__ bool keep_k(const PredDev &p, uint32_t x) {
     if (K == kAndMaskEq0) return (x & p.a) == 0u;
     if (K == kLt) return x < p.a;
     if (K == kPopcOdd) return (popc32(x) & 1u) != 0u;
-    if (K == kModNe0) return !(((x & p.c) == 0u) && ((x >> p.d) * p.a) <= p.b);
+    if (K == kModNe0) return rotr32(x * p.a, p.s) > p.b;
     if (K == kNe) return x != p.a;
     return true;
 }
@@ -193,6 +205,21 @@ __device__ __forceinline__ uint32_t mask4_k(const PredDev &p, uint32_t x0, uint3
     return uint32_t(keep_k<K>(p, x0)) | (uint32_t(keep_k<K>(p, x1)) << 1) |
            (uint32_t(keep_k<K>(p, x2)) << 2) | (uint32_t(keep_k<K>(p, x3)) << 3);
 }
+
+// Several compactions in a row as one: entry x is multiplied by op[0].mul and
+// tested, what passes is multiplied by op[1].mul and tested, and so on; an
+// entry is kept when it passes every test, with its last value. (Compacting
+// the compacted array keeps the same entries in the same order as keeping
+// those that pass both tests.) mul_all is the product of the multipliers.
+constexpr uint32_t kChainMax = 4;
+struct PredChain {
+    uint32_t n;
+    uint32_t mul_all;
+    struct {
+        PredDev pred;
+        uint32_t mul;
+    } op[kChainMax];
+};
 
 // Keep-mask of four consecutive entries (bit j = entry j kept). The switch is
 // on a value uniform across the block, so it costs one uniform branch per

@@ -107,6 +107,22 @@ ka_status launch_compact(const CompactLaunch &L, cudaStream_t stream);
 bool compact_tma_eligible(const CompactLaunch &L);
 ka_status launch_compact_tma(const CompactLaunch &L, cudaStream_t stream);
 
+// A chain of compactions in one pass over one array of n entries, or over the
+// interleave of two (in2 set: n counts pairs, both arrays 16-byte aligned),
+// at most kChainEntries entries in all. Workspace as for launch_compact.
+struct ChainLaunch {
+    const uint32_t *in, *in2;
+    uint32_t *out;
+    const uint32_t *n_ptr;
+    uint32_t *count;
+    uint64_t n;  // live length (in pairs with in2), or capacity when n_ptr is set
+    PredChain chain;
+    void *ws;
+    uint64_t ws_bytes;
+};
+constexpr uint64_t kChainEntries = 0xFFFFFFFCull;
+ka_status launch_compact_chain(const ChainLaunch &L, cudaStream_t stream);
+
 // The warp-specialised TMA kernel in scan mode (TMA shapes).
 ka_status launch_scan_tma(const uint32_t *in, uint64_t n, const uint32_t *n_ptr, uint32_t *out, uint32_t *total,
                           void *ws, uint64_t ws_bytes, ka_tile tile, cudaStream_t stream);

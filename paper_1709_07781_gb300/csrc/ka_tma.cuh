@@ -81,13 +81,109 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 constexpr int kSeg = 512;         // entries per compute warp and tile (32 lanes x 4 rows x 4)
 
 
-// The 4-entry keep mask for predicate kind PK (-1: the kind in p, chosen at
-// run time).
-template <int PK>
-__device__ __forceinline__ uint32_t mask4_of(const PredDev &p, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
-    if constexpr (PK < 0) return pred_mask4(p, x0, x1, x2, x3);
-    else if constexpr (PK == kAll) return 0xFu;
-    else return mask4_k<PK>(p, x0, x1, x2, x3);
+// Keep mask of a lane's 16 entries (entry c of row r: bit 4 r + c) and, above
+// it, the kept entries of each row (row r: bits 16 + 4 r .. 19 + 4 r), both by
+// one addition under the test's predicate: two instructions an entry for most
+// kinds. (Bool values shifted into place cost three to four, and the counts
+// four population counts more.)
+template <int K>
+__device__ __forceinline__ uint32_t tally(const PredDev &p, const uint32_t (&v)[4][4]) {
+    if constexpr (K == kAll) return 0x4444FFFFu;
+    uint32_t t[4] = {0u, 0u, 0u, 0u};
+    auto add = [&](auto keep) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint32_t one = (1u << (4 * r + c)) | (1u << (16 + 4 * r));
+                if constexpr (K == kPopcOdd)
+                    // (in one piece: the low bit goes straight to a predicate)
+                    asm("{\n .reg .pred q;\n .reg .b32 b;\n and.b32 b, %1, 1;\n setp.ne.u32 q, b, 0;\n"
+                        " @q add.u32 %0, %0, %2;\n}"
+                        : "+r"(t[r])
+                        : "r"(uint32_t(__popc(v[r][c]))), "r"(one));
+                else if (keep(v[r][c]))
+                    t[r] += one;
+            }
+    };
+    if (K == kModNe0 && p.s == 0u) add([&](uint32_t x) { return x * p.a > p.b; });  // odd divisors: no rotation
+    else add([&](uint32_t x) { return keep_k<K>(p, x); });
+    return (t[0] + t[1]) + (t[2] + t[3]);
+}
+
+// The tally of a keep mask alone.
+__device__ __forceinline__ uint32_t tally_of(uint32_t mask) {
+    uint32_t t = mask;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) t += uint32_t(__popc(mask & (0xFu << (4 * r)))) << (16 + 4 * r);
+    return t;
+}
+
+// Applies a chain to a lane's entries: v becomes the last values; the tally of
+// those that pass every test. The kind is switched on once per test for all
+// of the lane's entries.
+__device__ __forceinline__ uint32_t chain_tally(const PredChain &ch, uint32_t (&v)[4][4]) {
+    // (unrolled: every parameter is then read at a fixed place, as an operand)
+    uint32_t m = 0xFFFFu;
+#pragma unroll
+    for (uint32_t i = 0; i < kChainMax; ++i) {
+        if (i >= ch.n) break;
+        const PredDev &p = ch.op[i].pred;
+        if (ch.op[i].mul != 1u) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[r][c] *= ch.op[i].mul;
+        }
+        switch (p.kind) {
+        case kAndMaskEq0: m &= tally<kAndMaskEq0>(p, v); break;
+        case kLt: m &= tally<kLt>(p, v); break;
+        case kPopcOdd: m &= tally<kPopcOdd>(p, v); break;
+        case kModNe0: m &= tally<kModNe0>(p, v); break;
+        case kNe: m &= tally<kNe>(p, v); break;
+        default: break;
+        }
+    }
+    return tally_of(m);
+}
+
+// The tally cut to entries [vlo, vhi) of the segment.
+__device__ __forceinline__ uint32_t cut_tally(uint32_t t, uint32_t vlo, uint32_t vhi, int lane) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const uint32_t e0 = uint32_t(r * 128 + lane * 4);
+        const uint32_t skip = vlo > e0 ? min(vlo - e0, 4u) : 0u;
+        const uint32_t left = vhi > e0 ? vhi - e0 : 0u;
+        m |= (((0xFu << skip) & (left >= 4 ? 0xFu : ((1u << left) - 1u))) & 0xFu) << (4 * r);
+    }
+    return tally_of(t & m);
+}
+
+// Ranks of a lane's kept entries from its tally. The row counts, in 8-bit
+// fields (a row of the warp keeps at most 128), are scanned across the warp:
+// byte r of `excl` counts the kept entries of row r in the lanes before this
+// one, byte r of `rows` those of the whole row; `total` is the segment's. The
+// shuffle's own in-range predicate guards each addition.
+struct Ranks {
+    uint32_t excl, rows, total;
+};
+__device__ __forceinline__ Ranks rank_tally(uint32_t t) {
+    uint32_t packed = ((t >> 16) * 0x101u) & 0x00FF00FFu;  // nibbles to bytes
+    packed = (packed * 0x11u) & 0x0F0F0F0Fu;
+    uint32_t incl = packed;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1)
+        asm volatile(
+            "{\n .reg .pred q;\n .reg .b32 t;\n shfl.sync.up.b32 t|q, %0, %1, 0, 0xffffffff;\n"
+            " @q add.u32 %0, %0, t;\n}"
+            : "+r"(incl)
+            : "r"(d));
+    Ranks k;
+    k.excl = incl - packed;
+    k.rows = __shfl_sync(kFull, incl, 31);
+    k.total = __dp4a(k.rows, 0x01010101u, 0u);
+    return k;
 }
 
 // One warp counts the kept entries of its 512-entry segment (entries
@@ -96,12 +192,10 @@ __device__ __forceinline__ uint32_t mask4_of(const PredDev &p, uint32_t x0, uint
 template <int PK>
 __device__ __forceinline__ uint32_t compact_segment(uint32_t *seg, const PredDev &pred, uint32_t mul, uint32_t vlo,
                                                     uint32_t vhi, int lane) {
-    constexpr int ROWS = 4;
-    uint32_t v[ROWS][4], m[ROWS], packed = 0;
+    uint32_t v[4][4];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        const uint32_t e0 = uint32_t(r * 128 + lane * 4);
-        const uint4 q = *reinterpret_cast<const uint4 *>(seg + e0);
+    for (int r = 0; r < 4; ++r) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(seg + r * 128 + lane * 4);
         v[r][0] = q.x;
         v[r][1] = q.y;
         v[r][2] = q.z;
@@ -109,38 +203,25 @@ __device__ __forceinline__ uint32_t compact_segment(uint32_t *seg, const PredDev
     }
     if (mul != 1u) {
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r)
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int c = 0; c < 4; ++c) v[r][c] *= mul;
     }
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        const uint32_t e0 = uint32_t(r * 128 + lane * 4);
-        uint32_t mk = mask4_of<PK>(pred, v[r][0], v[r][1], v[r][2], v[r][3]);
-        if (vlo != 0u || vhi != uint32_t(kSeg)) {
-            const uint32_t skip = vlo > e0 ? min(vlo - e0, 4u) : 0u;
-            const uint32_t left = vhi > e0 ? vhi - e0 : 0u;
-            mk &= (0xFu << skip) & (left >= 4 ? 0xFu : ((1u << left) - 1u));
-        }
-        m[r] = mk;
-        packed += uint32_t(__popc(mk)) << (8 * r);
-    }
-    // per-row counts, 8 bits each (a row of the warp keeps at most 128)
-    const uint32_t incl = warp_incl_scan(packed, lane);
-    const uint32_t excl = incl - packed;
-    const uint32_t rows = __shfl_sync(kFull, incl, 31);
+    uint32_t t = tally<PK>(pred, v);
+    if (vlo != 0u || vhi != uint32_t(kSeg)) t = cut_tally(t, vlo, vhi, lane);
+    const Ranks k = rank_tally(t);
     __syncwarp();  // every lane holds its entries before any is overwritten
     uint32_t rowbase = 0;
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        uint32_t pos = rowbase + ((excl >> (8 * r)) & 0xFFu);
+    for (int r = 0; r < 4; ++r) {
+        uint32_t pos = rowbase + ((k.excl >> (8 * r)) & 0xFFu);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            if ((m[r] >> c) & 1u) seg[pos++] = v[r][c];
+            if ((t >> (4 * r + c)) & 1u) seg[pos++] = v[r][c];
         }
-        rowbase += (rows >> (8 * r)) & 0xFFu;
+        rowbase += (k.rows >> (8 * r)) & 0xFFu;
     }
-    return rowbase;
+    return k.total;
 }
 
 // One warp copies cnt compacted entries from shared memory (16-byte aligned)
@@ -191,6 +272,16 @@ __device__ __forceinline__ void warp_copy_out(const uint32_t *src, uint32_t *dst
     }
     const uint32_t t0 = head + 4 * body;
     if (uint32_t(lane) < cnt - t0) dst[t0 + lane] = src[t0 + lane];
+}
+
+// One warp writes cnt entries out of its ring (RW words, a power of two;
+// the entries start at word q), one per lane: few enough that realigning them
+// to 16 bytes would take more instructions than it saves.
+template <uint32_t RW>
+__device__ __forceinline__ void warp_ring_out(const uint32_t *ring, uint32_t q, uint32_t *dst, uint32_t cnt,
+                                              int lane) {
+#pragma unroll 1
+    for (uint32_t i = uint32_t(lane); i < cnt; i += 32) dst[i] = ring[(q + i) & (RW - 1u)];
 }
 
 }  // namespace tma

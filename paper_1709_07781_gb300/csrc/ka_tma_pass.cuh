@@ -33,16 +33,12 @@
 //   * scan: every segment is written out whole, from its stage, LAG tiles
 //     after it was scanned (the "prefix" mbarrier says its offset is ready),
 //     and only then is the stage released. One round trip per tile.
-//   * compaction: a warp whose segment keeps at most kSpillCap entries
-//     compacts them into a slot of its own small spill ring, releases the
-//     stage at once, and writes the entries out NS - 1 tiles later (one store
-//     per lane). A segment that keeps more is compacted in place in its stage
-//     and written out by its warp LAG tiles later, as in the scan. When every
-//     segment of the oldest pending tile was spilled, the look-back warp
-//     resolves every tile counted so far (up to BMAX) in one round trip; when
-//     one was held, it resolves that tile alone, whose write-out waits for it.
-//     At low selectivity the stages thus turn over at the rate of the copies,
-//     and the look-back's round trips overlap them instead of gating them.
+//   * compaction: a block that keeps few entries moves them out of the stage
+//     into a ring of kept entries per warp and releases the stage at once; one
+//     that keeps many holds them in the stage until they are written out (see
+//     tma_compact_pass). While the oldest pending tile keeps little, the
+//     look-back resolves every tile counted so far (up to BMAX) in one round
+//     trip; otherwise that tile alone, whose write-out waits for it.
 // One lane per warp arrives on an mbarrier, after __syncwarp: 32 arrivals on
 // one barrier word serialise. Every wait is bounded (a few seconds); on
 // time-out the kernel records a device error and still finishes.
@@ -65,16 +61,29 @@ struct TmaArgs {
     uint32_t lead;     // 0..3 entries before the input's first entry
     uint32_t out_vec;  // scan: out - lead is 16-byte aligned (output entries align with input entries)
     PredDev pred;
+    // the chain kernels (PK == kChainKind): their tests, and for an
+    // interleaved input its second array
+    const uint32_t *in2;
+    PredChain chain;
 };
 
-// Entries a compaction segment may keep and still go to the spill ring. At
-// 1 % kept a 512-entry segment keeps about 5 (more than 16 about once in
-// 10^4 segments); 16 rather than 32 leaves room in shared memory for a larger
-// tile, and a segment that keeps more takes the held path.
-constexpr int kSpillCap = 16;
+// Predicate kind of the kernels that run a chain of tests (TmaArgs::chain).
+constexpr int kChainKind = -1;
+
+// Kept entries of a segment up to which they are stored one by one.
+constexpr uint32_t kFewKept = 20;
+// Kept entries a pending tile up to which four, or two, are written out at a
+// time; and ring words kept free beyond what the last tile took.
+constexpr uint32_t kGroup4 = 64, kGroup2 = 100, kMargin = 32;
+
+// Offset of a tile's segments when its look-back gave up (no segment that
+// keeps an entry can start there: counts are at most 2^32 - 1).
+constexpr uint32_t kNoOffset = 0xFFFFFFFFu;
 
 // Block set-up shared by both passes (thread 0): the live length, the spin
 // limit and the launch epoch (one ticket per block; the last block resets).
+// With INTER, n and *n_ptr count pairs: the input has twice as many entries.
+template <bool INTER = false>
 __device__ __forceinline__ void tma_block_setup(const TmaArgs &a, uint32_t *s_n, uint32_t *s_spin,
                                                 uint32_t *s_epoch) {
     uint32_t n = a.n;
@@ -82,7 +91,7 @@ __device__ __forceinline__ void tma_block_setup(const TmaArgs &a, uint32_t *s_n,
         const uint32_t d = *a.n_ptr;
         n = d < n ? d : n;
     }
-    *s_n = n;
+    *s_n = INTER ? 2u * n : n;
     const uint32_t sl = a.ws->spin_limit;
     *s_spin = sl ? sl : kDefaultSpinLimit;
     uint32_t ep;
@@ -361,34 +370,123 @@ __device__ __forceinline__ void tma_scan_pass(const TmaArgs &a) {
 }
 
 // ====================================================================== compaction
-// Fused compaction with predicate kind PK (a PredKind, or -1: any kind,
-// chosen at run time): CWW compute warps (tile = CWW * 512 entries), S
-// stages, at most MAXG blocks, NS tile slots (counts, offsets, barriers, and
-// the NS slots of kSpillCap entries of each warp's spill ring), at most BMAX
-// tiles resolved per round trip of the look-back. A held segment is written
-// out LAG tiles after it was counted, a spilled one NS - 1 tiles after.
-template <int PK, int CWW, int S, int LAG, int MAXG, int NS, int BMAX>
+// Fused compaction with predicate kind PK (a PredKind, or kChainKind: the
+// tests of a.chain, one after the other): CWW compute warps (tile = CWW * 512
+// entries), at most MAXG blocks, NS tile slots (counts, offsets, barriers), at
+// most BMAX tiles resolved per round trip of the look-back.
+//
+// Shared memory holds SH tiles. A block uses them in one of two ways, chosen
+// by what its first tile keeps:
+//   * ring (at most kRingNum / kRingDen of the entries kept): SR stages, and
+//     the other SH - SR tiles as one ring of kept entries per compute warp. A
+//     warp moves the kept entries of its segment into its ring, releases the
+//     stage at once, and writes tiles out when the ring or the tile slots run
+//     out of room. So every stage is in flight or being counted, and the
+//     look-back has many tiles of time. What bounds it is the compute warps'
+//     instructions (250-340 a segment, 68 % of the issue slots), so tiles that
+//     keep little are written out four or two at a time.
+//   * hold (more kept): SH stages; a segment is compacted in place in its
+//     stage and written out LAG tiles later, and SH - LAG stages are in
+//     flight. What bounds it is HBM (0.98-1.01 of the copy rate). Above a
+//     fifth kept it is the faster of the two (17 % kept: ring 215 us, hold
+//     220 us; 25 %: 240 us and 218 us).
+// Both are correct for any data; a block whose first tile misleads it is only
+// slower. A chain, whose tests are instructions too, holds from
+// kRingNumChain / kRingDen.
+//
+// N = 2^28, shape (768, 16), s = 1 / 5 / 10 / 25 / 50 / 99 % kept, us: 164 /
+// 178 / 193 / 218 / 242 / 310. Before, four stages of 26 segments, each held
+// until its write-out unless every segment of the tile kept at most 16
+// entries: 175 / 207 / 212 / 230 / 266 / 331 (one stage in flight).
+//
+// A segment's count is posted before its entries are stored: the other blocks
+// wait for it. A warp waits for an older tile's offset only after it has
+// posted every tile up to that one, so no two blocks wait for each other.
+//
+// INTER: the input is the interleave of two arrays of a.n entries (entry 2i is
+// a.in[i], entry 2i + 1 is a.in2[i]; both 16-byte aligned, a.lead 0) that
+// exists nowhere in memory: a stage holds half a tile of each array, warp w's
+// segment is 256 entries of either half, and a held segment is compacted into
+// its own 256 words of the first half, then of the second.
+constexpr uint32_t kRingNum = 3, kRingNumChain = 2, kRingDen = 16;
+
+// The producer warp's loop of a compaction block (lane 0 only): as
+// tma_produce, for SR stages or SH, whichever the compute warps choose after
+// the first tile (the first SR tiles go to the same stages either way).
+template <int SR, int SH, int T, bool INTER>
+__device__ __forceinline__ void compact_produce(const TmaArgs &a, uint32_t *stage_mem, uint64_t *full_bar,
+                                                uint64_t *empty_bar, uint64_t *mode_bar, const uint32_t *s_ring,
+                                                uint32_t my_tiles, uint32_t full_tiles) {
+    const uint32_t G = gridDim.x, b = blockIdx.x;
+    uint32_t issued = 0, stages = SR, s = 0, lap = 0;  // tile jj: stage s = jj % stages, lap = jj / stages
+    for (uint32_t jj = 0; jj < my_tiles; ++jj) {
+        const uint32_t tile = b + jj * G;
+        if (tile >= full_tiles) break;
+        if (jj == uint32_t(SR)) {
+            if (!mbar_wait(mode_bar, 0u)) {
+                record_error(a.ws, kDevErrTimeout, tile);
+                break;
+            }
+            if (*s_ring == 0u) {
+                stages = SH;
+                s = SR;
+                lap = 0;
+            }
+        }
+        if (lap != 0u && !mbar_wait(&empty_bar[s], (lap - 1u) & 1u)) {
+            record_error(a.ws, kDevErrTimeout, tile);
+            break;
+        }
+        // the status sector of this block's tile two ahead: in L2 before its
+        // aggregate is stored and polled (first touches by those went to
+        // DRAM; 1 % faster at s = 1 %)
+        if (jj + 2 < my_tiles) prefetch_l2(status_at(a.status, uint64_t(tile) + 2u * G));
+        fence_proxy_async();  // the compute warps' accesses to this stage precede the copy into it
+        mbar_expect_tx(&full_bar[s], uint32_t(T) * 4u);
+        // two copies of half a tile each, both completing on the stage's
+        // barrier (measured 0.5 % faster than one at 1 % and 50 % kept)
+        static_assert(T % 8 == 0, "each half is whole 16-byte chunks");
+        const uint32_t *const h0 = INTER ? a.in + size_t(tile) * (T / 2) : a.in + size_t(tile) * T;
+        const uint32_t *const h1 = INTER ? a.in2 + size_t(tile) * (T / 2) : h0 + T / 2;
+        bulk_g2s(stage_mem + size_t(s) * T, h0, uint32_t(T / 2) * 4u, &full_bar[s]);
+        bulk_g2s(stage_mem + size_t(s) * T + T / 2, h1, uint32_t(T / 2) * 4u, &full_bar[s]);
+        issued = jj + 1;
+        if (++s == stages) {
+            s = 0;
+            ++lap;
+        }
+    }
+    // waits (bounded) for the last copies, so none lands after the block exits
+    for (uint32_t jj = issued > stages ? issued - stages : 0u; jj < issued; ++jj)
+        mbar_wait(&full_bar[jj % stages], (jj / stages) & 1u);
+}
+
+template <int PK, int CWW, int SR, int SH, int LAG, int MAXG, int NS, int BMAX, bool INTER = false>
 __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
-    constexpr int T = CWW * kSeg, ROWS = 4, SPC = kSpillCap, LAGS = NS - 1;
+    constexpr int T = CWW * kSeg, ROWS = 4, HALF = kSeg / 2;
+    constexpr uint32_t RW = uint32_t(SH - SR) * kSeg;  // words of a warp's ring
     constexpr int KB = (MAXG - 1 + 31) / 32;  // loads per lane for the G - 1 words before one tile
     static_assert(NS >= 2 && (NS & (NS - 1)) == 0, "tile slots: a power of two");
-    static_assert(LAG >= 1 && LAG < S && LAG <= LAGS, "a held segment is written out before its stage is refilled");
+    static_assert(SR >= 2 && SH > SR && (RW & (RW - 1)) == 0 && RW >= kSeg, "a ring: a power of two, one segment fits");
+    static_assert(LAG >= 1 && LAG < SH && LAG < NS, "a held segment is written out before its stage is refilled");
     static_assert(BMAX >= 1 && BMAX <= NS, "a batch of tiles fits the tile slots");
     static_assert(CWW <= 32, "the look-back warp holds one segment count per lane");
     static_assert(CWW * kSeg < 65536, "a tile aggregate fits the 16 low bits of s_pack");
+    static_assert(kSeg < 65536 && RW <= 65536, "count and ring word of a segment share a word");
+    static_assert(!INTER || PK == kChainKind, "an interleaved input is compacted by a chain");
     extern __shared__ __align__(128) uint32_t stage_mem[];
-    uint32_t *const spill_mem = stage_mem + size_t(S) * T;  // [CWW][NS][SPC]
-    __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], count_bar[NS], prefix_bar[NS];
-    __shared__ uint32_t s_wcnt[NS][CWW], s_woff[NS][CWW], s_err[NS];
+    __shared__ __align__(8) uint64_t full_bar[SH], empty_bar[SH], count_bar[NS], prefix_bar[NS], mode_bar;
+    __shared__ uint32_t s_wcnt[NS][CWW];  // per tile slot: segment counts (low half; above: first ring word)
+    __shared__ uint32_t s_woff[NS][CWW];  // per tile slot: segment offsets in the output
     __shared__ uint32_t s_pack[NS];  // per tile slot: (segments counted << 16) | kept so far
-    __shared__ uint32_t s_n, s_epoch, s_spin;
+    __shared__ uint32_t s_n, s_epoch, s_spin, s_ring;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t G = gridDim.x, b = blockIdx.x;
 
     if (tid == 0) {
-        tma_block_setup(a, &s_n, &s_spin, &s_epoch);
-        for (int s = 0; s < S; ++s) {
+        tma_block_setup<INTER>(a, &s_n, &s_spin, &s_epoch);
+        for (int s = 0; s < SH; ++s) {
             mbar_init(&full_bar[s], 1);
             mbar_init(&empty_bar[s], CWW);
         }
@@ -397,6 +495,8 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
             mbar_init(&count_bar[k], CWW);
             mbar_init(&prefix_bar[k], 1);
         }
+        mbar_init(&mode_bar, 1);
+        s_ring = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -414,9 +514,12 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     }
     const uint32_t my_tiles = live > b ? (live - b + G - 1) / G : 0u;
     uint64_t *const agg_words = a.status;  // entry per tile
+    if (my_tiles == 0) return;
 
     if (warp == CWW + 1) {
-        if (lane == 0) tma_produce<S, T>(a, stage_mem, full_bar, empty_bar, my_tiles, full_tiles);
+        if (lane == 0)
+            compact_produce<SR, SH, T, INTER>(a, stage_mem, full_bar, empty_bar, &mode_bar, &s_ring, my_tiles,
+                                              full_tiles);
         return;
     }
 
@@ -441,17 +544,18 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 // releases the waiters on this tile (once it is counted, so
                 // that the barriers' phases stay in step); its output is not
                 // written
-                if (lane == 0) s_err[k0] = 1u;
+                if (lane < CWW) s_woff[k0][lane] = kNoOffset;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&prefix_bar[k0]);
                 ++r;
                 continue;
             }
-            // Batching pays when the compute warps run ahead (every segment of
-            // tile r spilled); when some were held, their write-outs wait for
-            // this tile alone, and a batch would only lengthen the trip.
-            const uint32_t wc0 = lane < CWW ? s_wcnt[k0][lane] : 0u;
-            const bool held0 = __any_sync(kFull, wc0 > uint32_t(SPC));
+            // Batching pays when the compute warps run ahead (a ring that
+            // holds every tile slot's entries); when segments keep more, their
+            // write-outs wait for this tile alone, and a batch would only
+            // lengthen the trip.
+            const uint32_t wc0 = lane < CWW ? s_wcnt[k0][lane] & 0xFFFFu : 0u;
+            const bool held0 = __any_sync(kFull, wc0 > RW / uint32_t(NS - 1));
             uint32_t m = 1;
             while (!held0 && m < uint32_t(BMAX) && r + m < my_tiles &&
                    mbar_test_wait(&count_bar[(r + m) & uint32_t(NS - 1)], ((r + m) / NS) & 1u))
@@ -469,7 +573,7 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 for (int t = 0; t < BMAX; ++t) {
                     if (uint32_t(t) < m) {
                         const uint32_t k = (r + uint32_t(t)) & uint32_t(NS - 1);
-                        const uint32_t wc = lane < CWW ? s_wcnt[k][lane] : 0u;
+                        const uint32_t wc = lane < CWW ? s_wcnt[k][lane] & 0xFFFFu : 0u;
                         const uint32_t wincl = warp_incl_scan(wc, lane);
                         wexcl[t] = wincl - wc;
                         wagg[t] = __shfl_sync(kFull, wincl, 31);
@@ -554,10 +658,7 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                     const uint32_t prefix = before + part, agg = wagg[t];
                     before = prefix + agg;
                     if (lane < CWW) s_woff[k][lane] = prefix + wexcl[t];
-                    if (lane == 0) {
-                        s_err[k] = 0u;
-                        if (b + tt * G == live - 1) *a.count = prefix + agg;
-                    }
+                    if (lane == 0 && b + tt * G == live - 1) *a.count = prefix + agg;
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&prefix_bar[k]);  // offsets of tile tt ready
                 }
@@ -569,124 +670,257 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     }
 
     // ---------------------------------------------------------------- compute warps
-    // Iteration j: write out this warp's segment of tile j - LAG if it was
-    // held in its stage, and release that stage; write out its segment of
-    // tile j - (NS - 1) if that one was spilled; then count the segment of
-    // tile j and compact it into slot j % NS of the warp's spill ring (at
-    // most kSpillCap kept: the stage is released at once) or in place (held).
-    // Every segment's write-out waits for its tile's offsets, so slot j % NS
-    // (the last tile there is j - NS) is free when tile j is counted.
     const int w = warp;
     const uint32_t mul = a.mul;
-    uint32_t *const seg_base = stage_mem + w * kSeg;
-    uint32_t *const spill_base = spill_mem + size_t(w) * NS * SPC;
+    uint32_t *const seg_base = stage_mem + w * (INTER ? HALF : kSeg);
     const uint32_t lead_tiles = a.lead != 0u ? 1u : 0u;  // tile 0 starts before the input
-    for (uint32_t j = 0; j < my_tiles + uint32_t(LAGS); ++j) {
-        if (j >= uint32_t(LAG) && j - uint32_t(LAG) < my_tiles) {
-            const uint32_t jp = j - uint32_t(LAG), k = jp & uint32_t(NS - 1);
-            const uint32_t cnt = s_wcnt[k][w];
-            if (cnt > uint32_t(SPC)) {
-                const int s = int(jp % S);
-                const bool ok = mbar_wait(&prefix_bar[k], (jp / NS) & 1u);
-                if (!ok && lane == 0) record_error(a.ws, kDevErrTimeout, b + jp * G);
-                const uint32_t off = s_woff[k][w];
-                __syncwarp();
-                if (ok && s_err[k] == 0u) warp_copy_out(seg_base + size_t(s) * T, a.out + off, cnt, lane);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty_bar[s]);  // this warp is done with the stage
-            }
-        }
-        if (j >= uint32_t(LAGS)) {
-            const uint32_t jq = j - uint32_t(LAGS), k = jq & uint32_t(NS - 1);
-            const uint32_t cnt = s_wcnt[k][w];
-            if (cnt <= uint32_t(SPC)) {
-                const bool ok = mbar_wait(&prefix_bar[k], (jq / NS) & 1u);
-                if (!ok && lane == 0) record_error(a.ws, kDevErrTimeout, b + jq * G);
-                if (ok && s_err[k] == 0u && uint32_t(lane) < cnt) a.out[s_woff[k][w] + lane] = spill_base[k * SPC + lane];
-            }
-        }
-        if (j < my_tiles) {
-            const uint32_t tile = b + j * G, k = j & uint32_t(NS - 1);
-            const int s = int(j % S);
-            uint32_t *seg = seg_base + size_t(s) * T;
-            // Entries [vlo, vhi) of this segment are input entries: all of them
-            // except in the first tile of an input with lead entries and in
-            // the ragged last tile, the only tiles that compute the bounds
-            // (64-bit position: the last tile's later segments can lie past
-            // 2^32 when T does not divide 2^32). The ragged tile is read with
-            // plain loads (zeros outside the input).
-            uint32_t vlo = 0u, vhi = uint32_t(kSeg);
-            const bool full_tile = tile < full_tiles;
-            if (!full_tile || tile < lead_tiles) {
-                const uint64_t base = uint64_t(tile) * T + uint32_t(w) * kSeg;
-                vlo = base < a.lead ? a.lead - uint32_t(base) : 0u;
-                vhi = n > base ? uint32_t(min(n - base, uint64_t(kSeg))) : 0u;
-                if (!full_tile) {
+
+    // Segment of iteration j (tile `tile`, stage s) in shared memory, its
+    // entries [vlo, vhi) being input entries: all of them except in the first
+    // tile of an input with lead entries and in the ragged last tile, the only
+    // tiles that compute the bounds (64-bit position: the last tile's later
+    // segments can lie past 2^32 when T does not divide 2^32). The ragged tile
+    // is read with plain loads (zeros outside the input).
+    uint32_t vlo, vhi;
+    auto arrive = [&](uint32_t tile, uint32_t *seg, int s, uint32_t parity) {
+        vlo = 0u;
+        vhi = uint32_t(kSeg);
+        const bool full_tile = tile < full_tiles;
+        if (!full_tile || tile < lead_tiles) {
+            const uint64_t base = uint64_t(tile) * T + uint32_t(w) * kSeg;
+            vlo = base < a.lead ? a.lead - uint32_t(base) : 0u;
+            vhi = n > base ? uint32_t(min(n - base, uint64_t(kSeg))) : 0u;
+            if (!full_tile) {
+                if constexpr (INTER) {
+                    // (base is even, and so is vhi: whole pairs)
+                    const uint64_t pair = base / 2;
+                    for (uint32_t e = uint32_t(lane); e < uint32_t(HALF); e += 32) {
+                        seg[e] = 2u * e < vhi ? a.in[pair + e] : 0u;
+                        seg[T / 2 + e] = 2u * e < vhi ? a.in2[pair + e] : 0u;
+                    }
+                } else {
                     const uint32_t *src = a.in + base;
                     for (uint32_t e = uint32_t(lane); e < uint32_t(kSeg); e += 32)
                         seg[e] = e >= vlo && e < vhi ? src[e] : 0u;
-                    __syncwarp();
                 }
+                __syncwarp();
             }
-            if (full_tile && !mbar_wait(&full_bar[s], (j / S) & 1u) && lane == 0)
-                record_error(a.ws, kDevErrTimeout, tile);
-            const bool edge = vlo != 0u || vhi != uint32_t(kSeg);
-            uint32_t v[ROWS][4], mk4[ROWS], packed = 0;
+        }
+        if (full_tile && !mbar_wait(&full_bar[s], parity) && lane == 0) record_error(a.ws, kDevErrTimeout, tile);
+    };
+    // The segment's entries (after the transform) and their ranks.
+    uint32_t v[ROWS][4], tl;
+    auto count = [&](const uint32_t *seg) -> Ranks {
 #pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const uint32_t e0 = uint32_t(r * 128 + lane * 4);
+        for (int r = 0; r < ROWS; ++r) {
+            const uint32_t e0 = uint32_t(r * 128 + lane * 4);
+            if constexpr (INTER) {
+                const uint2 p = *reinterpret_cast<const uint2 *>(seg + e0 / 2);
+                const uint2 q = *reinterpret_cast<const uint2 *>(seg + T / 2 + e0 / 2);
+                v[r][0] = p.x;
+                v[r][1] = q.x;
+                v[r][2] = p.y;
+                v[r][3] = q.y;
+            } else {
                 const uint4 q = *reinterpret_cast<const uint4 *>(seg + e0);
                 v[r][0] = q.x;
                 v[r][1] = q.y;
                 v[r][2] = q.z;
                 v[r][3] = q.w;
             }
+        }
+        if constexpr (PK == kChainKind) {
+            tl = chain_tally(a.chain, v);
+        } else {
             if (mul != 1u) {
 #pragma unroll
                 for (int r = 0; r < ROWS; ++r)
 #pragma unroll
                     for (int c = 0; c < 4; ++c) v[r][c] *= mul;
             }
-#pragma unroll
-            for (int r = 0; r < ROWS; ++r) {
-                const uint32_t e0 = uint32_t(r * 128 + lane * 4);
-                uint32_t mk = mask4_of<PK>(a.pred, v[r][0], v[r][1], v[r][2], v[r][3]);
-                if (edge) {
-                    const uint32_t skip = vlo > e0 ? min(vlo - e0, 4u) : 0u;
-                    const uint32_t left = vhi > e0 ? vhi - e0 : 0u;
-                    mk &= (0xFu << skip) & (left >= 4 ? 0xFu : ((1u << left) - 1u));
+            tl = tally<PK>(a.pred, v);
+        }
+        if (vlo != 0u || vhi != uint32_t(kSeg)) tl = cut_tally(tl, vlo, vhi, lane);
+        return rank_tally(tl);
+    };
+    // Posts the count of iteration j's segment, whose entries start at word p
+    // of the warp's ring. The last segment counted publishes the tile aggregate
+    // at once, and that of the block's first tile decides how the block uses
+    // its memory. (A warp of its own that waits for the counts and publishes
+    // takes the atomic's round trip off the compute warps, but publishes later:
+    // 241 -> 248 us at N = 2^28 and 50 % kept.)
+    auto post = [&](uint32_t j, uint32_t tile, uint32_t total, uint32_t p) {
+        if (lane == 0) {
+            const uint32_t k = j & uint32_t(NS - 1);
+            s_wcnt[k][w] = p << 16 | total;
+            const uint32_t prev = atomicAdd(&s_pack[k], (1u << 16) | total);
+            if ((prev >> 16) == uint32_t(CWW - 1)) {
+                const uint32_t agg = (prev & 0xFFFFu) + total;
+                s_pack[k] = 0;
+                st_relaxed_u64(status_at(agg_words, tile), pack_status(epoch, kFlagAggregate, agg));
+                if (j == 0) {
+                    s_ring = agg * kRingDen <= uint32_t(T) * (PK == kChainKind ? kRingNumChain : kRingNum) ? 1u : 0u;
+                    mbar_arrive(&mode_bar);
                 }
-                mk4[r] = mk;
-                packed += uint32_t(__popc(mk)) << (8 * r);
             }
-            // per-row counts, 8 bits each (a row of the warp keeps at most 128)
-            const uint32_t incl = warp_incl_scan(packed, lane);
-            const uint32_t excl = incl - packed;
-            const uint32_t rows = __shfl_sync(kFull, incl, 31);
-            const uint32_t total = (rows & 0xFFu) + ((rows >> 8) & 0xFFu) + ((rows >> 16) & 0xFFu) + (rows >> 24);
-            const bool spilled = total <= uint32_t(SPC);
-            if (spilled) {
-                // At most kSpillCap entries for the whole warp: each lane
-                // stores only its own kept entries, in order, reading each
-                // back from the stage (as many trips as the busiest lane has
-                // kept entries; at low selectivity most lanes hold none, where
-                // the 16 predicated stores below cost every lane 16 slots).
-                // Entry r * 128 + 4 lane + c of the segment is bit 4 r + c of
-                // the lane's mask; its slot is the lane's first slot in row r
-                // (byte r of `first`: the rows before r plus the lanes before
-                // this one in row r; every count is at most 16, so no byte
-                // carries) plus its kept entries in row r already stored.
-                const uint32_t orig = mk4[0] | (mk4[1] << 4) | (mk4[2] << 8) | (mk4[3] << 12);
-                const uint32_t first = excl + rows * 0x01010100u;
-                uint32_t *const ring = spill_base + k * SPC;
-                const uint32_t *const mine = seg + uint32_t(lane) * 4u;
-                for (uint32_t m = orig; m != 0u; m &= m - 1u) {
-                    const uint32_t i = uint32_t(__ffs(int(m))) - 1u, r = i >> 2;
-                    const uint32_t pos = ((first >> (8u * r)) & 0xFFu) + __popc((orig ^ m) & (0xFu << (4u * r)));
-                    ring[pos] = mine[r * 128u + (i & 3u)] * mul;
+            mbar_arrive(&count_bar[k]);
+        }
+    };
+    // Offset of iteration j's segment once its tile is resolved (kNoOffset:
+    // the look-back gave up).
+    auto offset = [&](uint32_t j) -> uint32_t {
+        const uint32_t k = j & uint32_t(NS - 1);
+        if (!mbar_wait(&prefix_bar[k], (j / NS) & 1u)) {
+            if (lane == 0) record_error(a.ws, kDevErrTimeout, b + j * G);
+            return kNoOffset;
+        }
+        return s_woff[k][w];
+    };
+
+    arrive(b, seg_base, 0, 0u);
+    post(0, b, count(seg_base).total, 0u);
+    if (!mbar_wait(&mode_bar, 0u) && lane == 0) record_error(a.ws, kDevErrTimeout, b);
+
+    if (s_ring != 0u) {
+        // -------------------------------------------------------------- ring
+        // Tile jq is the oldest one not written out; `used` ring words are
+        // taken, and the next entries go to word p. A tile's entries start on
+        // a 16-byte boundary.
+        uint32_t *const ring = stage_mem + size_t(SR) * T + size_t(w) * RW;
+        uint32_t jq = 0, p = 0, used = 0, last = 0, s = 0, parity = 0;
+        auto flush = [&]() {  // the oldest tile
+            const uint32_t c = s_wcnt[jq & uint32_t(NS - 1)][w], cnt = c & 0xFFFFu, off = offset(jq);
+            if (off != kNoOffset) warp_ring_out<RW>(ring, c >> 16, a.out + off, cnt, lane);
+            __syncwarp();  // read before the ring's words are written again
+            used -= (cnt + 3u) & ~3u;
+            ++jq;
+        };
+        // The oldest N, 32 / N lanes each (tiles are resolved in order: the
+        // last one's offset comes last): one wait and one chain of dependent
+        // loads where there would be N.
+        auto flush_group = [&](auto group) {
+            constexpr uint32_t N = decltype(group)::value, LANES = 32u / N;
+            const uint32_t k = (jq + uint32_t(lane) / LANES) & uint32_t(NS - 1);
+            const uint32_t c = s_wcnt[k][w], cnt = c & 0xFFFFu;
+            if (offset(jq + N - 1u) != kNoOffset) {
+                const uint32_t off = s_woff[k][w];
+                if (off != kNoOffset) {
+                    uint32_t *const dst = a.out + off;
+                    const uint32_t q = c >> 16;
+#pragma unroll 1
+                    for (uint32_t i = uint32_t(lane) % LANES; i < cnt; i += 2u * LANES) {
+                        const uint32_t i2 = i + LANES;
+                        const uint32_t x = ring[(q + i) & (RW - 1u)], x2 = ring[(q + i2) & (RW - 1u)];
+                        dst[i] = x;
+                        if (i2 < cnt) dst[i2] = x2;
+                    }
+                }
+            }
+            uint32_t room = (cnt + 3u) & ~3u;
+#pragma unroll
+            for (uint32_t d = LANES; d < 32u; d *= 2u) room += __shfl_xor_sync(kFull, room, d);
+            __syncwarp();  // read before the ring's words are written again
+            used -= room;
+            jq += N;
+        };
+        uint32_t tile = b;
+        for (uint32_t j = 0; j < my_tiles; ++j, tile += G) {
+            // tile j's slot, and room for a tile that keeps a little more than
+            // the last; several tiles at once while they are small (the
+            // youngest of them has had three tiles' time to be resolved)
+            while (j - jq >= uint32_t(NS) || (jq < j && used + last + kMargin > RW)) {
+                const uint32_t pend = j - jq;
+                if (NS >= 8 && pend >= 7u && used <= pend * kGroup4) flush_group(std::integral_constant<uint32_t, 4>{});
+                else if (NS >= 8 && pend >= 5u && used <= pend * kGroup2) flush_group(std::integral_constant<uint32_t, 2>{});
+                else flush();
+            }
+            uint32_t *const seg = seg_base + size_t(s) * T;
+            if (j != 0) arrive(tile, seg, int(s), parity);
+            Ranks rk = count(seg);
+            if (j != 0) post(j, tile, rk.total, p);
+            const uint32_t room = (rk.total + 3u) & ~3u;
+            while (used + room > RW) {  // it keeps more than the last: make room, then count it again
+                flush();
+                rk = count(seg);
+            }
+            if (rk.total <= kFewKept) {
+                // Few entries for the whole warp: each lane stores only its
+                // own kept entries, in order, reading each back from the stage
+                // (as many trips as the busiest lane has kept entries; most
+                // lanes hold none, where the 16 predicated stores below cost
+                // every lane 16 slots). Entry r * 128 + 4 lane + c of the
+                // segment is bit 4 r + c of the lane's mask; its place is the
+                // lane's first in row r (byte r of `first`: the rows before r
+                // plus the lanes before this one in row r; no byte carries)
+                // plus its kept entries in row r already stored.
+                const uint32_t orig = tl & 0xFFFFu;
+                const uint32_t first = rk.excl + rk.rows * 0x01010100u;
+                const uint32_t *const mine = seg + uint32_t(lane) * (INTER ? 2u : 4u);
+                for (uint32_t left = orig; left != 0u; left &= left - 1u) {
+                    const uint32_t i = uint32_t(__ffs(int(left))) - 1u, r = i >> 2;
+                    const uint32_t pos =
+                        ((first >> (8u * r)) & 0xFFu) + __popc((orig ^ left) & (0xFu << (4u * r)));
+                    const uint32_t x = INTER ? mine[r * 64u + ((i >> 1) & 1u) + (i & 1u) * uint32_t(T / 2)]
+                                             : mine[r * 128u + (i & 3u)];
+                    ring[(p + pos) & (RW - 1u)] = x * mul;
+                }
+            } else {
+                const uint32_t dst = smem_addr(ring);
+                auto store = [&](auto wrap) {  // wrap: p + total passes the ring's end
+                    uint32_t rowbase = p;
+#pragma unroll
+                    for (int r = 0; r < ROWS; ++r) {
+                        uint32_t pos = rowbase + ((rk.excl >> (8 * r)) & 0xFFu);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            if ((tl >> (4 * r + c)) & 1u) {
+                                st_shared_u32(dst + 4u * (wrap ? pos & (RW - 1u) : pos), v[r][c]);
+                                ++pos;
+                            }
+                        }
+                        rowbase += (rk.rows >> (8 * r)) & 0xFFu;
+                    }
+                };
+                if (p + rk.total <= RW) store(std::false_type{});
+                else store(std::true_type{});
+            }
+            p = (p + room) & (RW - 1u);
+            used += room;
+            last = room;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty_bar[s]);  // nothing of this tile is left in the stage
+            if (++s == uint32_t(SR)) {
+                s = 0;
+                parity ^= 1u;
+            }
+        }
+        while (jq < my_tiles) flush();
+    } else {
+        // -------------------------------------------------------------- hold
+        uint32_t s = 0, parity = 0, so = 0;  // stages of tiles j and j - LAG
+        uint32_t tile = b;
+        for (uint32_t j = 0; j < my_tiles + uint32_t(LAG); ++j, tile += G) {
+            if (j >= uint32_t(LAG)) {
+                const uint32_t jp = j - uint32_t(LAG), cnt = s_wcnt[jp & uint32_t(NS - 1)][w] & 0xFFFFu,
+                               off = offset(jp);
+                if (off != kNoOffset) {
+                    const uint32_t *const held = seg_base + size_t(so) * T;
+                    if constexpr (INTER) {
+                        warp_copy_out(held, a.out + off, min(cnt, uint32_t(HALF)), lane);
+                        if (cnt > uint32_t(HALF)) warp_copy_out(held + T / 2, a.out + off + HALF, cnt - HALF, lane);
+                    } else {
+                        warp_copy_out(held, a.out + off, cnt, lane);
+                    }
                 }
                 __syncwarp();
-            } else {
+                if (lane == 0) mbar_arrive(&empty_bar[so]);  // this warp is done with the stage
+                if (++so == uint32_t(SH)) so = 0;
+            }
+            if (j < my_tiles) {
+                uint32_t *const seg = seg_base + size_t(s) * T;
+                if (j != 0) arrive(tile, seg, int(s), parity);
+                const Ranks rk = count(seg);
+                if (j != 0) post(j, tile, rk.total, 0u);
                 // in place, at the front of the segment (an explicit st.shared
                 // to the segment's shared-memory address)
                 const uint32_t dst = smem_addr(seg);
@@ -694,34 +928,33 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 uint32_t rowbase = 0;
 #pragma unroll
                 for (int r = 0; r < ROWS; ++r) {
-                    uint32_t pos = rowbase + ((excl >> (8 * r)) & 0xFFu);
+                    uint32_t pos = rowbase + ((rk.excl >> (8 * r)) & 0xFFu);
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        if ((mk4[r] >> c) & 1u) st_shared_u32(dst + 4u * pos++, v[r][c]);
+                        if ((tl >> (4 * r + c)) & 1u) {
+                            if constexpr (INTER)
+                                st_shared_u32(dst + 4u * pos + (pos >= uint32_t(HALF) ? 4u * (T / 2 - HALF) : 0u),
+                                              v[r][c]);
+                            else
+                                st_shared_u32(dst + 4u * pos, v[r][c]);
+                            ++pos;
+                        }
                     }
-                    rowbase += (rows >> (8 * r)) & 0xFFu;
+                    rowbase += (rk.rows >> (8 * r)) & 0xFFu;
                 }
                 __syncwarp();
-            }
-            if (lane == 0) {
-                s_wcnt[k][w] = total;
-                // the last segment counted publishes the tile aggregate at once
-                const uint32_t prev = atomicAdd(&s_pack[k], (1u << 16) | total);
-                if ((prev >> 16) == uint32_t(CWW - 1)) {
-                    s_pack[k] = 0;
-                    st_relaxed_u64(status_at(agg_words, tile),
-                                   pack_status(epoch, kFlagAggregate, (prev & 0xFFFFu) + total));
+                if (++s == uint32_t(SH)) {
+                    s = 0;
+                    parity ^= 1u;
                 }
-                mbar_arrive(&count_bar[k]);
-                if (spilled) mbar_arrive(&empty_bar[s]);  // nothing of this tile is left in the stage
             }
         }
     }
 }
 
-template <int PK, int CWW, int S, int LAG, int MAXG, int MINB, int NS, int BMAX>
+template <int PK, int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX, bool INTER = false>
 __global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_compact_tma(const TmaArgs a) {
-    tma_compact_pass<PK, CWW, S, LAG, MAXG, NS, BMAX>(a);
+    tma_compact_pass<PK, CWW, SR, SH, LAG, MAXG, NS, BMAX, INTER>(a);
 }
 
 template <int CWW, int S, int LAG, int MAXG, int MINB>
@@ -761,40 +994,55 @@ ka_status launch_tma_kernel(Kern kern, PerDeviceInt &grid_cache, size_t smem, co
     return cuda_status(cudaLaunchKernelEx(&cfg, kern, a));
 }
 
-template <int PK, int CWW, int S, int LAG, int MAXG, int MINB, int NS, int BMAX>
+template <int PK, int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX, bool INTER = false>
 ka_status launch_compact_shape(const TmaArgs &a, uint64_t cap, cudaStream_t stream) {
     constexpr int BLOCK = (CWW + 2) * 32, T = CWW * kSeg;
-    const size_t smem = size_t(S) * T * 4 + size_t(CWW) * NS * kSpillCap * 4;
+    const size_t smem = size_t(SH) * T * 4;
     static PerDeviceInt grid_cache;
-    return launch_tma_kernel<BLOCK, T, MAXG>(k_compact_tma<PK, CWW, S, LAG, MAXG, MINB, NS, BMAX>, grid_cache, smem,
-                                             a, cap, stream);
+    return launch_tma_kernel<BLOCK, T, MAXG>(k_compact_tma<PK, CWW, SR, SH, LAG, MAXG, MINB, NS, BMAX, INTER>, grid_cache,
+                                             smem, a, cap, stream);
 }
 
-// One configuration's kernels: the scan, or the compaction for predicate kind
-// pk (every kind has its own kernel).
-template <int CWW, int S, int LAG, int MAXG, int MINB, int NS, int BMAX>
-ka_status launch_tma_config(const TmaArgs &a, bool scan, int32_t pk, uint64_t cap, cudaStream_t stream) {
-    if (scan) {
-        constexpr int BLOCK = (CWW + 2) * 32, T = CWW * kSeg;
-        static PerDeviceInt grid_cache;
-        return launch_tma_kernel<BLOCK, T, MAXG>(k_scan_tma<CWW, S, LAG, MAXG, MINB>, grid_cache,
-                                                 size_t(S) * T * 4, a, cap, stream);
-    }
+// The chain's kernels of a configuration: one array, or the interleave of two.
+template <int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX>
+ka_status launch_chain_config(const TmaArgs &a, uint64_t cap, cudaStream_t stream) {
+    if (a.in2) return launch_compact_shape<kChainKind, CWW, SR, SH, LAG, MAXG, MINB, NS, BMAX, true>(a, cap, stream);
+    return launch_compact_shape<kChainKind, CWW, SR, SH, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
+}
+
+// One configuration's compaction for predicate kind pk (every kind has its
+// own kernel).
+template <int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX>
+ka_status launch_compact_config(const TmaArgs &a, int32_t pk, uint64_t cap, cudaStream_t stream) {
     switch (pk) {
-    case kAndMaskEq0: return launch_compact_shape<kAndMaskEq0, CWW, S, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
-    case kLt: return launch_compact_shape<kLt, CWW, S, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
-    case kPopcOdd: return launch_compact_shape<kPopcOdd, CWW, S, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
-    case kModNe0: return launch_compact_shape<kModNe0, CWW, S, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
-    case kNe: return launch_compact_shape<kNe, CWW, S, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
-    case kAll: return launch_compact_shape<kAll, CWW, S, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
-    default: return launch_compact_shape<-1, CWW, S, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
+#define KA_CASE(K) \
+    case K: return launch_compact_shape<K, CWW, SR, SH, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
+        KA_CASE(kAndMaskEq0)
+        KA_CASE(kLt)
+        KA_CASE(kPopcOdd)
+        KA_CASE(kModNe0)
+        KA_CASE(kNe)
+        KA_CASE(kAll)
+#undef KA_CASE
+    default: return KA_E_ARG;
     }
+}
+
+// One configuration's scan.
+template <int CWW, int S, int LAG, int MAXG, int MINB>
+ka_status launch_scan_config(const TmaArgs &a, uint64_t cap, cudaStream_t stream) {
+    constexpr int BLOCK = (CWW + 2) * 32, T = CWW * kSeg;
+    static PerDeviceInt grid_cache;
+    return launch_tma_kernel<BLOCK, T, MAXG>(k_scan_tma<CWW, S, LAG, MAXG, MINB>, grid_cache, size_t(S) * T * 4, a,
+                                             cap, stream);
 }
 
 // One translation unit per tile shape instantiates its configuration.
 ka_status launch_tma_768(const TmaArgs &a, bool scan, int32_t pk, uint64_t cap, cudaStream_t stream);
 ka_status launch_tma_512(const TmaArgs &a, bool scan, int32_t pk, uint64_t cap, cudaStream_t stream);
 ka_status launch_tma_256(const TmaArgs &a, bool scan, int32_t pk, uint64_t cap, cudaStream_t stream);
+ka_status launch_chain_768(const TmaArgs &a, uint64_t cap, cudaStream_t stream);
+ka_status launch_chain_512(const TmaArgs &a, uint64_t cap, cudaStream_t stream);
 
 }  // namespace tma
 }  // namespace ka
