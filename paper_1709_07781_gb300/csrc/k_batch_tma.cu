@@ -297,30 +297,64 @@ __global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_batch_tma(const BatchA
             const uint32_t base = uint32_t(w) * kSeg;
             const uint32_t vlo = ti.vlo > base ? ti.vlo - base : 0u;
             const uint32_t vhi = ti.vhi > base ? min(ti.vhi - base, uint32_t(kSeg)) : 0u;
-            uint32_t rowbase = 0;
+            uint32_t v[4][4], tl = 0;
             if (vhi > vlo) {
-                // the tile's item fixes the predicate: one branch per tile into
-                // a count loop made for that predicate kind
-                switch (ti.pred.kind) {
-                case kAndMaskEq0: rowbase = compact_segment<kAndMaskEq0>(seg, ti.pred, mul, vlo, vhi, lane); break;
-                case kLt: rowbase = compact_segment<kLt>(seg, ti.pred, mul, vlo, vhi, lane); break;
-                case kPopcOdd: rowbase = compact_segment<kPopcOdd>(seg, ti.pred, mul, vlo, vhi, lane); break;
-                case kModNe0: rowbase = compact_segment<kModNe0>(seg, ti.pred, mul, vlo, vhi, lane); break;
-                case kNe: rowbase = compact_segment<kNe>(seg, ti.pred, mul, vlo, vhi, lane); break;
-                default: rowbase = compact_segment<kAll>(seg, ti.pred, mul, vlo, vhi, lane); break;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint4 q = *reinterpret_cast<const uint4 *>(seg + r * 128 + lane * 4);
+                    v[r][0] = q.x;
+                    v[r][1] = q.y;
+                    v[r][2] = q.z;
+                    v[r][3] = q.w;
                 }
+                if (mul != 1u) {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) v[r][c] *= mul;
+                }
+                // the tile's item fixes the predicate: one branch per tile into
+                // a count made for that predicate kind
+                switch (ti.pred.kind) {
+                case kAndMaskEq0: tl = tally<kAndMaskEq0>(ti.pred, v); break;
+                case kLt: tl = tally<kLt>(ti.pred, v); break;
+                case kPopcOdd: tl = tally<kPopcOdd>(ti.pred, v); break;
+                case kModNe0: tl = tally<kModNe0>(ti.pred, v); break;
+                case kNe: tl = tally<kNe>(ti.pred, v); break;
+                default: tl = tally<kAll>(ti.pred, v); break;
+                }
+                if (vlo != 0u || vhi != uint32_t(kSeg)) tl = cut_tally(tl, vlo, vhi, lane);
             }
+            const Ranks rk = rank_tally(tl);
+            // posted before the entries are stored: the other blocks wait for
+            // the count (and the last segment counted publishes the aggregate)
             if (lane == 0) {
-                s_wcnt[k][w] = rowbase;
-                const uint32_t prev = atomicAdd(&s_pack[k], (1u << 16) | rowbase);
+                s_wcnt[k][w] = rk.total;
+                const uint32_t prev = atomicAdd(&s_pack[k], (1u << 16) | rk.total);
                 if ((prev >> 16) == uint32_t(CWW - 1)) {
                     s_pack[k] = 0;
                     st_relaxed_u64(status_at(agg_words, tile),
-                                   pack_status(epoch, kFlagAggregate, (prev & 0xFFFFu) + rowbase));
+                                   pack_status(epoch, kFlagAggregate, (prev & 0xFFFFu) + rk.total));
                 }
+                mbar_arrive(&count_bar[k]);
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&count_bar[k]);
+            __syncwarp();  // every lane holds its entries before any is overwritten
+            // in place, at the front of the segment
+            const uint32_t dst = smem_addr(seg);
+            uint32_t rowbase = dst;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                uint32_t at = rowbase + 4u * ((rk.excl >> (8 * r)) & 0xFFu);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if ((tl >> (4 * r + c)) & 1u) {
+                        st_shared_u32(at, v[r][c]);
+                        at += 4u;
+                    }
+                }
+                rowbase += 4u * ((rk.rows >> (8 * r)) & 0xFFu);
+            }
+            __syncwarp();  // stored before another lane writes them out
         }
     }
 }

@@ -186,44 +186,6 @@ __device__ __forceinline__ Ranks rank_tally(uint32_t t) {
     return k;
 }
 
-// One warp counts the kept entries of its 512-entry segment (entries
-// [vlo, vhi) are input entries; the others are ignored) and compacts them in
-// place at the segment's front, in order. Returns the count.
-template <int PK>
-__device__ __forceinline__ uint32_t compact_segment(uint32_t *seg, const PredDev &pred, uint32_t mul, uint32_t vlo,
-                                                    uint32_t vhi, int lane) {
-    uint32_t v[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(seg + r * 128 + lane * 4);
-        v[r][0] = q.x;
-        v[r][1] = q.y;
-        v[r][2] = q.z;
-        v[r][3] = q.w;
-    }
-    if (mul != 1u) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[r][c] *= mul;
-    }
-    uint32_t t = tally<PK>(pred, v);
-    if (vlo != 0u || vhi != uint32_t(kSeg)) t = cut_tally(t, vlo, vhi, lane);
-    const Ranks k = rank_tally(t);
-    __syncwarp();  // every lane holds its entries before any is overwritten
-    uint32_t rowbase = 0;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        uint32_t pos = rowbase + ((k.excl >> (8 * r)) & 0xFFu);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            if ((t >> (4 * r + c)) & 1u) seg[pos++] = v[r][c];
-        }
-        rowbase += (k.rows >> (8 * r)) & 0xFFu;
-    }
-    return k.total;
-}
-
 // One warp copies cnt compacted entries from shared memory (16-byte aligned)
 // to dst (4-byte aligned): single entries up to dst's next 16-byte boundary,
 // then 16-byte stores, each assembled from two aligned 16-byte shared loads,
