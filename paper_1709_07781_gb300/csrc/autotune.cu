@@ -40,12 +40,39 @@ const ka_tile kTmaOnlyShapes[] = {{768, 16}};
 const ka_tile kBatchOnlyShapes[] = {{704, 16}};
 
 ka_tile default_tile(int32_t kernel, uint64_t n) {
-    if (kernel == KA_KERNEL_COMPACT && n >= (1ull << 22)) return ka_tile{768, 16};  // TMA kernel
+    if (kernel == KA_KERNEL_COMPACT) {
+        // Per call among others in a CUDA graph, us, 1 % / 50 % kept:
+        //   n        (256, 4)     (256, 8)     (256, 16)    (512, 16)    (768, 16)
+        //   2^12     2.7 / 3.5    2.7 / 3.4    4.0 / 4.4    6.2 / 6.9    6.7 / 7.4
+        //   2^16     4.2 / 4.2    3.4 / 3.9    4.8 / 5.0    4.4 / 4.9    6.6 / 7.0
+        //   2^18     5.2 / 5.4    3.9 / 4.0    4.3 / 5.3    4.5 / 5.1    6.7 / 6.9
+        //   2^19     6.4 / 6.1    5.7 / 5.6    4.3 / 4.8    4.3 / 4.7    6.8 / 7.1
+        //   2^20     7.7 / 7.9    6.0 / 6.3    5.4 / 5.6    4.4 / 4.8    6.6 / 6.9
+        //   2^21     12.6 / 12.9  7.5 / 8.0    8.1 / 8.3    6.5 / 7.4    6.8 / 7.2
+        //   2^23     34.8 / 37.1  21.0 / 22.7  13.0 / 14.2  10.1 / 12.4  10.9 / 11.5
+        // A register shape runs as the wave kernel while every tile of it runs
+        // at once (see k_compact.cu); the TMA shapes' set-up pays from where
+        // that kernel's status words and stores add up. (Up to 2^20 the default
+        // keeps to tiles of at most 4096 entries.)
+        if (n >= (1ull << 22)) return ka_tile{768, 16};
+        if (n > (1ull << 20)) return ka_tile{512, 16};
+        if (n >= 3ull << 17) return ka_tile{256, 16};
+        return n >= (1ull << 13) ? ka_tile{256, 8} : ka_tile{256, 4};
+    }
     if (kernel == KA_KERNEL_BATCH) return ka_tile{704, 16};                         // TMA batch kernel
     if (kernel == KA_KERNEL_SCAN && n >= (1ull << 22)) return ka_tile{512, 16};      // TMA kernel, scan mode
     if (n >= (1ull << 24)) return ka_tile{256, 16};
     if (n >= (1ull << 21)) return ka_tile{256, 8};
     return ka_tile{256, 4};
+}
+
+// Entries a tile that the workspace of a call without a tile has to be sized
+// for: no more than this, whatever shape the call then uses.
+uint32_t default_workspace_tile(int32_t kernel, uint64_t n) {
+    const ka_tile t = default_tile(kernel, n);
+    const uint32_t te = t.block * t.ipt;
+    if (kernel != KA_KERNEL_COMPACT || n >= (1ull << 22)) return te;
+    return n >= (1ull << 21) ? 2048u : 1024u;
 }
 
 bool save_table(const char *path) {
@@ -133,6 +160,15 @@ ka_tile resolve_tile(int32_t kernel, uint64_t n, const ka_tile *requested) {
     if (kernel != KA_KERNEL_BATCH && !tile_supported(t.block, t.ipt) && n > 0xFFFFFFFCull) t = ka_tile{512, 16};
     memo[memo_next++ & 3u] = Memo{gen, kernel, n, t};  // (tagged with the generation read before the lookup)
     return t;
+}
+
+uint64_t workspace_tiles(int32_t kernel, uint64_t n, const ka_tile *requested) {
+    if (requested && requested->block && requested->ipt) return 0;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (g_table.count({kernel, bucket_of(n)})) return 0;
+    }
+    return tiles_for(n, default_workspace_tile(kernel, n));
 }
 
 // Times `launch` over `reps` runs after `warm` untimed runs; returns the median

@@ -5,8 +5,14 @@
 // Blocks are persistent (grid = resident blocks) and take tiles by ticket.
 // Output offsets never exceed input positions, so out == in is safe: a tile
 // writes only after all its predecessors have loaded their input.
+//
+// An array whose tiles all run at once (up to about 2 M entries) has a kernel of
+// its own, k_compact_wave: such a call is a chain of latencies, not of bytes.
+#include <algorithm>
+
 #include "ka_internal.h"
 #include "ka_tile.cuh"
+#include "ka_tma.cuh"
 
 namespace ka {
 
@@ -70,6 +76,204 @@ __global__ void __launch_bounds__(BLOCK) k_compact_fused(const CompactArgs a) {
     }
 }
 
+constexpr uint32_t kWaveMaxTiles = 1216;  // every tile reads a status word of each before it
+
+// One tile per block, every block running at once. What bounds it is the chain
+// ticket, loads, counts, offset, stores, a round trip to L2 or more each; so
+//   * a block loads the tile of its own index before its ticket is back, and
+//     only loads again if the ticket names another tile (tickets come in block
+//     order nearly always; they guarantee that every tile before this one is
+//     running). With a device length, the loads wait for the length;
+//   * a tile waits for no look-back of another: it adds up the counts of all
+//     tiles before it, one status word per thread, all in flight together,
+//     where a decoupled look-back walks 32 at a time and waits for prefixes;
+//   * warp w of a block owns 32 IPT consecutive entries, so one barrier of the
+//     warps' totals ranks the whole tile;
+//   * the tile starts on a 16-byte boundary of the input (up to 3 entries
+//     before it, in the same 16 bytes as its first, are read and ignored).
+// A ka_compact call among others in a CUDA graph, us, at 50 % kept, against the
+// ticketed kernel below in the same shape: (256, 4), 2^16 entries 5.3 -> 4.2,
+// 2^18 6.1 -> 5.4, 2^20 9.2 -> 7.9; (512, 8), 2^18 5.4 -> 4.9, 2^20 6.4 -> 5.4,
+// 2^21 8.7 -> 7.3.
+struct WaveArgs {
+    const uint32_t *in;  // input rounded down to 16 bytes: entry i of the input is in[lead + i]
+    uint32_t *out;
+    const uint32_t *n_ptr;
+    uint32_t *count;
+    WsHeader *ws;
+    uint64_t *status;
+    uint32_t n;
+    uint32_t status_cap;
+    uint32_t lead;
+    PredChain chain;
+};
+
+template <int BLOCK, int IPT>
+__global__ void __launch_bounds__(BLOCK) k_compact_wave(const WaveArgs a) {
+    constexpr int ROWS = IPT / 4, WARPS = BLOCK / 32, SEG = 32 * IPT;
+    constexpr uint32_t T = BLOCK * IPT;
+    static_assert(ROWS >= 1 && ROWS <= 4 && WARPS <= 32, "a lane's tally, and one warp scans the warps");
+    __shared__ uint32_t s_out[T];
+    __shared__ uint32_t s_wtot[WARPS], s_part[WARPS];
+    __shared__ uint32_t s_ticket, s_epoch, s_n, s_spin, s_bad;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+    uint32_t v[ROWS][4];
+    auto load = [&](uint32_t tile, uint32_t n) {  // n: entries from the 16-byte boundary
+        const uint64_t base = uint64_t(tile) * T + uint32_t(warp) * SEG;
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            const uint64_t e = base + uint32_t(r * 128 + lane * 4);
+            uint4 q = make_uint4(0u, 0u, 0u, 0u);
+            if (e < n) q = *reinterpret_cast<const uint4 *>(a.in + e);
+            v[r][0] = q.x;
+            v[r][1] = q.y;
+            v[r][2] = q.z;
+            v[r][3] = q.w;
+        }
+    };
+    if (!a.n_ptr) load(blockIdx.x, a.n + a.lead);
+    if (tid == 0) {
+        uint32_t ep;
+        bool last;
+        s_ticket = take_ticket(a.ws, 0u, &ep, &last);  // one ticket per block: the last one starts the next epoch
+        s_epoch = ep;
+        uint32_t n = a.n;
+        if (a.n_ptr) {
+            const uint32_t d = *a.n_ptr;
+            n = d < n ? d : n;
+        }
+        s_n = n;
+        const uint32_t sl = a.ws->spin_limit;
+        s_spin = sl ? sl : kDefaultSpinLimit;
+        s_bad = 0u;
+    }
+    __syncthreads();
+    const uint32_t n = s_n ? s_n + a.lead : 0u, tile = s_ticket, epoch = s_epoch;
+    const uint32_t live = (n + T - 1u) / T;
+    if (live > a.status_cap) {
+        if (tid == 0 && tile == 0u) record_error(a.ws, kDevErrWorkspace, 0);
+        return;
+    }
+    if (tile >= live) {
+        if (tid == 0 && live == 0u && tile == 0u) *a.count = 0u;
+        return;
+    }
+    if (a.n_ptr || tile != blockIdx.x) load(tile, n);
+
+    uint32_t tl = tma::chain_tally(a.chain, v);
+    {
+        const uint32_t base = tile * T + uint32_t(warp) * SEG;
+        const uint32_t vlo = base < a.lead ? a.lead - base : 0u;
+        const uint32_t vhi = n > base ? min(n - base, uint32_t(SEG)) : 0u;
+        if (vlo != 0u || vhi != uint32_t(SEG)) tl = tma::cut_tally(tl, vlo, vhi, lane);
+    }
+    const tma::Ranks rk = tma::rank_tally(tl);
+    if (lane == 0) s_wtot[warp] = rk.total;
+    __syncthreads();
+    const uint32_t wt = lane < WARPS ? s_wtot[lane] : 0u;
+    const uint32_t wincl = warp_incl_scan(wt, lane);
+    const uint32_t agg = __shfl_sync(kFull, wincl, 31);
+    if (tid == 0) st_relaxed_u64(status_at(a.status, tile), pack_status(epoch, kFlagAggregate, agg));
+
+    // the kept entries in tile order, while the other tiles' counts arrive
+    uint32_t rowbase = __shfl_sync(kFull, wincl - wt, warp);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        uint32_t pos = rowbase + ((rk.excl >> (8 * r)) & 0xFFu);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if ((tl >> (4 * r + c)) & 1u) s_out[pos++] = v[r][c];
+        rowbase += (rk.rows >> (8 * r)) & 0xFFu;
+    }
+
+    const uint32_t want = epoch & kEpochMask, spin = s_spin;
+    uint32_t sum = 0, polls = 0, sleep_ns = 0;
+    for (uint32_t i = uint32_t(tid); i < tile;) {
+        const uint64_t w = ld_relaxed_u64(status_at(a.status, i));
+        if (uint32_t(w >> 34) == want && (uint32_t(w >> 32) & 3u) == kFlagAggregate) {
+            sum += uint32_t(w);
+            i += BLOCK;
+            continue;
+        }
+        if (++polls >= spin) {
+            record_error(a.ws, kDevErrTimeout, tile);
+            s_bad = 1u;
+            break;
+        }
+        if (polls > 4) {
+            __nanosleep(sleep_ns);
+            sleep_ns = sleep_ns < 128 ? sleep_ns * 2 + 32 : 128;
+        }
+    }
+    sum = warp_sum(sum);
+    if (lane == 0) s_part[warp] = sum;
+    __syncthreads();
+    const uint32_t prefix = warp_sum(lane < WARPS ? s_part[lane] : 0u);
+    if (s_bad) return;  // (recorded; nothing of this tile is written)
+    if (tid == 0 && tile == live - 1u) *a.count = prefix + agg;
+    uint32_t *const dst = a.out + prefix;
+    for (uint32_t k = uint32_t(tid); k < agg; k += BLOCK) dst[k] = s_out[k];
+}
+
+template <int BLOCK, int IPT>
+static uint32_t wave_tiles() {  // tiles that run at once
+    static PerDeviceInt cache;
+    return uint32_t(per_device_value(cache, current_device(), [] {
+        int occ = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_compact_wave<BLOCK, IPT>, BLOCK, 0);
+        return occ > 0 ? occ * device_info().sm_count : 1;
+    }));
+}
+
+// The wave kernel of a register shape, if every tile of L runs at once.
+// KA_E_UNSUPPORTED: it does not.
+template <int BLOCK, int IPT>
+static ka_status launch_wave_shape(WaveArgs a, uint64_t cap, cudaStream_t stream) {
+    const uint64_t tiles = tiles_for(cap + a.lead, BLOCK * IPT);
+    if (tiles > wave_tiles<BLOCK, IPT>() || tiles > kWaveMaxTiles) return KA_E_UNSUPPORTED;
+    k_compact_wave<BLOCK, IPT><<<unsigned(tiles ? tiles : 1), BLOCK, 0, stream>>>(a);
+    return cuda_status(cudaGetLastError());
+}
+
+static ka_status launch_wave(const ChainLaunch &L, ka_tile t, cudaStream_t stream) {
+    if (L.n > uint64_t(kWaveMaxTiles) * t.block * t.ipt) return KA_E_UNSUPPORTED;
+    WaveArgs a{};
+    a.lead = uint32_t(reinterpret_cast<uintptr_t>(L.in) & 15u) / 4u;
+    a.in = L.in - a.lead;
+    a.out = L.out;
+    a.n_ptr = L.n_ptr;
+    a.count = L.count;
+    a.ws = static_cast<WsHeader *>(L.ws);
+    a.status = reinterpret_cast<uint64_t *>(static_cast<char *>(L.ws) + kWsHeaderBytes);
+    a.n = uint32_t(L.n);
+    a.status_cap = status_capacity(L.ws_bytes);
+    a.chain = L.chain;
+    switch (shape_key(t.block, t.ipt)) {
+#define KA_CASE(B, I) \
+    case shape_key(B, I): return launch_wave_shape<B, I>(a, L.n, stream);
+        KA_FOR_EACH_SHAPE(KA_CASE)
+#undef KA_CASE
+    default: return KA_E_UNSUPPORTED;
+    }
+}
+
+ka_status launch_compact_chain(const ChainLaunch &L, cudaStream_t stream) {
+    const uint64_t entries = L.in2 ? 2 * L.n : L.n;
+    if (entries > kChainEntries || L.chain.n == 0 || L.chain.n > kChainMax) return KA_E_ARG;
+    if (L.n && (!L.in || !L.out)) return KA_E_ARG;
+    if (!L.count || L.n_ptr == L.count) return KA_E_ARG;
+    if (L.in2 && ((reinterpret_cast<uintptr_t>(L.in) | reinterpret_cast<uintptr_t>(L.in2)) & 15u)) return KA_E_ARG;
+    ka_tile t = resolve_tile(KA_KERNEL_COMPACT, entries, nullptr);
+    if (!L.in2 && !tma_shape(t.block, t.ipt)) {
+        const ka_status ws_ok = check_workspace(L.ws, L.ws_bytes, tiles_for(entries, t.block * t.ipt));
+        if (ws_ok != KA_OK) return ws_ok;
+        const ka_status s = launch_wave(L, t, stream);
+        if (s != KA_E_UNSUPPORTED) return s;
+    }
+    return launch_chain_tma(L, t, stream);
+}
+
 template <int BLOCK, int IPT>
 static ka_status launch_shape(const CompactArgs &a, uint64_t cap, cudaStream_t stream) {
     constexpr int T = BLOCK * IPT;
@@ -94,11 +298,18 @@ ka_status launch_compact(const CompactLaunch &L, cudaStream_t stream) {
     if (L.n_ptr && L.n_ptr == L.count) return KA_E_ARG;
     const ka_tile t = L.tile;
     if (!tile_supported_for(KA_KERNEL_COMPACT, t.block, t.ipt)) return KA_E_ARG;
-    const uint64_t tiles = tiles_for(L.n, t.block * t.ipt);
+    const uint64_t tiles = std::max(L.ws_tiles, tiles_for(L.n, t.block * t.ipt));
     const ka_status ws_ok = check_workspace(L.ws, L.ws_bytes, tiles);
     if (ws_ok != KA_OK) return ws_ok;
     if (compact_tma_eligible(L)) return launch_compact_tma(L, stream);
     if (!tile_supported(t.block, t.ipt)) return KA_E_ARG;  // a TMA-only shape beyond its size limit
+    ChainLaunch one{L.in, nullptr, L.out, L.n_ptr, L.count, L.n, {}, L.ws, L.ws_bytes};
+    one.chain.n = 1;
+    one.chain.mul_all = L.mul;
+    one.chain.op[0].pred = L.pred;
+    one.chain.op[0].mul = L.mul;
+    const ka_status wave = launch_wave(one, t, stream);
+    if (wave != KA_E_UNSUPPORTED) return wave;
     CompactArgs a;
     a.in = L.in;
     a.out = L.out;
@@ -139,6 +350,7 @@ extern "C" ka_status ka_compact(const uint32_t *d_in, uint64_t n, const uint32_t
     L.mul = xform == KA_XFORM_HASH ? kHashMul : 1u;
     L.ws = d_ws;
     L.ws_bytes = ws_bytes;
+    L.ws_tiles = n <= 0xFFFFFFFFull ? workspace_tiles(KA_KERNEL_COMPACT, n, tile) : 0;
     L.tile = resolve_tile(KA_KERNEL_COMPACT, n, tile);
     return launch_compact(L, static_cast<cudaStream_t>(stream));
 }

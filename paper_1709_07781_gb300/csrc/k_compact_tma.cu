@@ -48,15 +48,9 @@ ka_status launch_compact_tma(const CompactLaunch &L, cudaStream_t stream) {
     return launch_tma(a, L.tile, false, L.pred.kind, L.n + a.lead, stream);
 }
 
-ka_status launch_compact_chain(const ChainLaunch &L, cudaStream_t stream) {
+ka_status launch_chain_tma(const ChainLaunch &L, ka_tile t, cudaStream_t stream) {
     const uint64_t entries = L.in2 ? 2 * L.n : L.n;
-    if (entries > kChainEntries || L.chain.n == 0 || L.chain.n > kChainMax) return KA_E_ARG;
-    if (L.n && (!L.in || !L.out)) return KA_E_ARG;
-    if (!L.count || L.n_ptr == L.count) return KA_E_ARG;
-    if (L.in2 && ((reinterpret_cast<uintptr_t>(L.in) | reinterpret_cast<uintptr_t>(L.in2)) & 15u)) return KA_E_ARG;
-    // the compaction's shape when it is one of the two that have chain
-    // kernels, else the smaller of those
-    ka_tile t = resolve_tile(KA_KERNEL_COMPACT, entries, nullptr);
+    // two of the shapes have chain kernels: the smaller of them for any other
     if (t.block != 768) t = ka_tile{512, 16};
     const ka_status ws_ok = check_workspace(L.ws, L.ws_bytes, tiles_for(entries, t.block * t.ipt));
     if (ws_ok != KA_OK) return ws_ok;
@@ -73,8 +67,8 @@ ka_status launch_compact_chain(const ChainLaunch &L, cudaStream_t stream) {
     a.status_cap = status_capacity(L.ws_bytes);
     a.mul = L.chain.mul_all;
     a.chain = L.chain;
-    return t.block == 768 ? launch_chain_768(a, entries + a.lead, stream)
-                          : launch_chain_512(a, entries + a.lead, stream);
+    const uint64_t cap = entries + a.lead;
+    return t.block == 768 ? launch_chain_768(a, cap, stream) : launch_chain_512(a, cap, stream);
 }
 
 ka_status launch_scan_tma(const uint32_t *in, uint64_t n, const uint32_t *n_ptr, uint32_t *out, uint32_t *total,

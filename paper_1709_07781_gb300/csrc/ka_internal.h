@@ -67,6 +67,11 @@ bool batch_tma_shape(uint32_t block, uint32_t ipt);
 bool tile_supported_for(int32_t kernel, uint32_t block, uint32_t ipt);
 // Shape to use for `kernel` at size n: explicit shape, else autotuned, else default.
 ka_tile resolve_tile(int32_t kernel, uint64_t n, const ka_tile *requested);
+// Tiles that the workspace of a call must hold when it leaves the shape to the
+// library's default (0: the call or the autotuner names a shape, whose own tile
+// count is what must fit). The default shape changes with what is fastest; the
+// workspace a caller has to bring does not.
+uint64_t workspace_tiles(int32_t kernel, uint64_t n, const ka_tile *requested);
 // The batch kernel has one shape for every batch, stored under this size.
 constexpr uint64_t kBatchTileKey = 1ull << 17;
 ka_status autotune_batch(uint64_t total, const char *cache_path, ka_tile *best, float *best_us, void *stream);
@@ -100,6 +105,7 @@ struct CompactLaunch {
     void *ws;
     uint64_t ws_bytes;
     ka_tile tile;
+    uint64_t ws_tiles = 0;  // tiles the workspace must hold, if more than the shape needs
 };
 ka_status launch_compact(const CompactLaunch &L, cudaStream_t stream);
 // The warp-specialised TMA kernel (the TMA shapes, any 4-byte-aligned input
@@ -122,6 +128,8 @@ struct ChainLaunch {
 };
 constexpr uint64_t kChainEntries = 0xFFFFFFFCull;
 ka_status launch_compact_chain(const ChainLaunch &L, cudaStream_t stream);
+// The TMA kernels' chain, for the shape t or the nearest that has one.
+ka_status launch_chain_tma(const ChainLaunch &L, ka_tile t, cudaStream_t stream);
 
 // The warp-specialised TMA kernel in scan mode (TMA shapes).
 ka_status launch_scan_tma(const uint32_t *in, uint64_t n, const uint32_t *n_ptr, uint32_t *out, uint32_t *total,

@@ -81,18 +81,18 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 constexpr int kSeg = 512;         // entries per compute warp and tile (32 lanes x 4 rows x 4)
 
 
-// Keep mask of a lane's 16 entries (entry c of row r: bit 4 r + c) and, above
-// it, the kept entries of each row (row r: bits 16 + 4 r .. 19 + 4 r), both by
+// Keep mask of a lane's entries (entry c of row r: bit 4 r + c) and, above it, the kept entries of each row (row r: bits 16 + 4 r .. 19 + 4 r), both by
 // one addition under the test's predicate: two instructions an entry for most
 // kinds. (Bool values shifted into place cost three to four, and the counts
 // four population counts more.)
-template <int K>
-__device__ __forceinline__ uint32_t tally(const PredDev &p, const uint32_t (&v)[4][4]) {
-    if constexpr (K == kAll) return 0x4444FFFFu;
+template <int K, int ROWS>
+__device__ __forceinline__ uint32_t tally(const PredDev &p, const uint32_t (&v)[ROWS][4]) {
+    static_assert(ROWS <= 4, "16 mask bits and four counts");
+    if constexpr (K == kAll) return 0x4444FFFFu & (0xFFFFu >> (16 - 4 * ROWS)) * 0x10001u;
     uint32_t t[4] = {0u, 0u, 0u, 0u};
     auto add = [&](auto keep) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < ROWS; ++r)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const uint32_t one = (1u << (4 * r + c)) | (1u << (16 + 4 * r));
@@ -122,16 +122,17 @@ __device__ __forceinline__ uint32_t tally_of(uint32_t mask) {
 // Applies a chain to a lane's entries: v becomes the last values; the tally of
 // those that pass every test. The kind is switched on once per test for all
 // of the lane's entries.
-__device__ __forceinline__ uint32_t chain_tally(const PredChain &ch, uint32_t (&v)[4][4]) {
+template <int ROWS>
+__device__ __forceinline__ uint32_t chain_tally(const PredChain &ch, uint32_t (&v)[ROWS][4]) {
     // (unrolled: every parameter is then read at a fixed place, as an operand)
-    uint32_t m = 0xFFFFu;
+    uint32_t m = 0xFFFFu >> (16 - 4 * ROWS);
 #pragma unroll
     for (uint32_t i = 0; i < kChainMax; ++i) {
         if (i >= ch.n) break;
         const PredDev &p = ch.op[i].pred;
         if (ch.op[i].mul != 1u) {
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            for (int r = 0; r < ROWS; ++r)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) v[r][c] *= ch.op[i].mul;
         }

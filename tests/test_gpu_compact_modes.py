@@ -93,3 +93,32 @@ def test_density_that_changes_from_segment_to_segment(ka, tile):
 @pytest.mark.parametrize("s", [0.01, 0.5])
 def test_tile_edges(ka, n, s):
     check(ka, with_density(n, s, n), (768, 16))
+
+
+@pytest.mark.parametrize("tile", [(128, 4), (256, 4), (128, 16), (512, 8), (1024, 8)])
+@pytest.mark.parametrize("off", [0, 1, 3])
+def test_arrays_whose_tiles_all_run_at_once(ka, tile, off):
+    """The wave kernel of the register shapes: one entry to a full wave and one
+    tile past it (the ticketed kernel), inputs at every word of 16 bytes,
+    device lengths below the capacity, every predicate kind, in place."""
+    t = tile[0] * tile[1]
+    wave = torch.cuda.get_device_properties(0).multi_processor_count * (2048 // tile[0])
+    for n in (1, t - 1, t, t + 1, 37 * t + 5, min(wave, 1216) * t - off, wave * t + t + 1):
+        x = ki.uniform_u32(n & 0xFFF, n)
+        buf = to_dev(np.concatenate([np.zeros(off, np.uint32), x]), pad=4)
+        for name, param, xform in (("lt", HALF, 0), ("mod_ne0", 12, 1), ("and_mask_eq0", 3, 0), ("popc_odd", 0, 1),
+                                   ("ne", int(x[0]), 0), ("lt", 0, 0)):
+            for live in (None, n // 2, 0):
+                ws = Workspace(ka, n, tile)
+                d_out, d_count = empty(n + 4), empty(1)
+                d_n = None if live is None else to_dev(np.array([live], np.uint32))
+                kind = getattr(ka, "KA_PRED_" + name.upper())
+                assert ka.ka_compact(buf.data_ptr() + 4 * off, n, d_n, kind, param, xform, d_out, d_count, ws.ptr,
+                                     ws.nbytes, tile, stream()) == 0
+                torch.cuda.synchronize()
+                want = x if live is None else x[:live]
+                y, k = oracle.compact(oracle.map_hash(want) if xform else want, name, param)
+                got = to_host(d_out)
+                assert word(d_count) == k and ws.status(ka) == 0
+                assert np.array_equal(got[:k], y) and (got[k:] == 0xDEADBEEF).all()
+        check(ka, x, tile, in_place=True)
