@@ -2,6 +2,8 @@
 // fused compaction and the exclusive scan for the TMA tile shapes, with any
 // 4-byte-aligned input (tiles are shifted back to a 16-byte boundary). The
 // kernels are instantiated in k_tma_<shape>.cu, one file per tile shape.
+#include <algorithm>
+
 #include "ka_tma_pass.cuh"
 
 namespace ka {
@@ -48,6 +50,70 @@ ka_status launch_compact_tma(const CompactLaunch &L, cudaStream_t stream) {
     return launch_tma(a, L.tile, false, L.pred.kind, L.n + a.lead, stream);
 }
 
+namespace {
+
+// A chain as something simpler with the same result: one test, or a set of
+// different ones. Products that come before every test may go in front of them
+// all; tests of one kind combine (two upper bounds are the lower of them) or, if
+// they do not, and where a product stands between or after tests, the chain
+// stays as it is (mask -1). mask 0: keep everything.
+struct Simplified {
+    int mask = -1;
+    uint32_t mul = 1;
+    PredSet set{};
+    PredDev one{};  // the test, when the mask has one bit or none
+};
+
+Simplified simplify(const PredChain &c) {
+    Simplified s;
+    s.one.kind = kAll;
+    int mask = 0;
+    for (uint32_t i = 0; i < c.n; ++i) {
+        const PredDev &p = c.op[i].pred;
+        if (c.op[i].mul != 1u) {
+            if (mask != 0) return s;
+            s.mul *= c.op[i].mul;
+        }
+        int bit = 0;
+        switch (p.kind) {
+        case kAndMaskEq0:
+            bit = kSetAnd;
+            s.set.and_mask |= p.a;
+            break;
+        case kLt:
+            bit = kSetLt;
+            s.set.lt = mask & bit ? std::min(s.set.lt, p.a) : p.a;
+            break;
+        case kPopcOdd: bit = kSetPopc; break;
+        case kModNe0:
+            bit = kSetMod;
+            if (mask & bit && (s.set.mod_a != p.a || s.set.mod_b != p.b || s.set.mod_s != p.s)) return s;
+            s.set.mod_a = p.a;
+            s.set.mod_b = p.b;
+            s.set.mod_s = p.s;
+            break;
+        case kNe:
+            bit = kSetNe;
+            if (mask & bit && s.set.ne != p.a) return s;
+            s.set.ne = p.a;
+            break;
+        default: continue;  // kAll
+        }
+        mask |= bit;
+        s.one = p;
+    }
+    if (mask == kSetAnd) s.one.a = s.set.and_mask;
+    if (mask == kSetLt) s.one.a = s.set.lt;
+    s.mask = mask;
+    return s;
+}
+
+}  // namespace
+
+// The chain kernel tests an entry with each op in turn, for any ops, at the cost
+// of a switch and a mask per op (16 entries: 20 to 30 instructions) and of two
+// to four instructions an entry; the kernels made for one test or for a set
+// only have the latter. Which is which is settled here, on the host.
 ka_status launch_chain_tma(const ChainLaunch &L, ka_tile t, cudaStream_t stream) {
     const uint64_t entries = L.in2 ? 2 * L.n : L.n;
     // two of the shapes have chain kernels: the smaller of them for any other
@@ -68,6 +134,21 @@ ka_status launch_chain_tma(const ChainLaunch &L, ka_tile t, cudaStream_t stream)
     a.mul = L.chain.mul_all;
     a.chain = L.chain;
     const uint64_t cap = entries + a.lead;
+    const Simplified s = simplify(L.chain);
+    if (s.mask >= 0) {
+        const bool single = (s.mask & (s.mask - 1)) == 0;
+        a.mul = s.mul;
+        a.pred = s.one;
+        a.set = s.set;
+        if (single && !L.in2) return launch_tma(a, t, false, s.one.kind, cap, stream);
+        if (single && t.block == 768) return launch_inter_768(a, s.one.kind, cap, stream);
+        if (!single && !L.in2 && t.block == 768)
+            for (auto sets : {launch_sets_768_a, launch_sets_768_b, launch_sets_768_c, launch_sets_768_d}) {
+                const ka_status r = sets(a, s.mask, cap, stream);
+                if (r != KA_E_UNSUPPORTED) return r;
+            }
+        a.mul = L.chain.mul_all;
+    }
     return t.block == 768 ? launch_chain_768(a, cap, stream) : launch_chain_512(a, cap, stream);
 }
 

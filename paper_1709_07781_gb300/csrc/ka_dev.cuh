@@ -221,6 +221,13 @@ struct PredChain {
     } op[kChainMax];
 };
 
+// A set of at least two different tests, which an entry has to pass all of:
+// bits of its mask (a kernel is made for each), and their parameters.
+enum SetBit : int { kSetAnd = 1, kSetLt = 2, kSetPopc = 4, kSetMod = 8, kSetNe = 16 };
+struct PredSet {
+    uint32_t and_mask, lt, mod_a, mod_b, mod_s, ne;
+};
+
 // Keep-mask of four consecutive entries (bit j = entry j kept). The switch is
 // on a value uniform across the block, so it costs one uniform branch per
 // four entries.

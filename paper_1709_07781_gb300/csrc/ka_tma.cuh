@@ -111,6 +111,28 @@ __device__ __forceinline__ uint32_t tally(const PredDev &p, const uint32_t (&v)[
     return (t[0] + t[1]) + (t[2] + t[3]);
 }
 
+// The tally for the set of tests MASK: the tests of an entry are one chain of
+// predicates, and only the last makes a bit and a count.
+template <int MASK, int ROWS>
+__device__ __forceinline__ uint32_t set_tally(const PredSet &p, const uint32_t (&v)[ROWS][4]) {
+    static_assert(ROWS <= 4, "16 mask bits and four counts");
+    uint32_t t[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const uint32_t x = v[r][c];
+            bool keep = true;
+            if (MASK & kSetAnd) keep = keep && (x & p.and_mask) == 0u;
+            if (MASK & kSetLt) keep = keep && x < p.lt;
+            if (MASK & kSetNe) keep = keep && x != p.ne;
+            if (MASK & kSetMod) keep = keep && rotr32(x * p.mod_a, p.mod_s) > p.mod_b;
+            if (MASK & kSetPopc) keep = keep && (__popc(x) & 1u) != 0u;
+            if (keep) t[r] += (1u << (4 * r + c)) | (1u << (16 + 4 * r));
+        }
+    return (t[0] + t[1]) + (t[2] + t[3]);
+}
+
 // The tally of a keep mask alone.
 __device__ __forceinline__ uint32_t tally_of(uint32_t mask) {
     uint32_t t = mask;

@@ -65,10 +65,12 @@ struct TmaArgs {
     // interleaved input its second array
     const uint32_t *in2;
     PredChain chain;
+    PredSet set;  // the set kernels' tests
 };
 
-// Predicate kind of the kernels that run a chain of tests (TmaArgs::chain).
-constexpr int kChainKind = -1;
+// Predicate kind of the kernels that run a chain of tests (TmaArgs::chain), and
+// of those made for a set of tests (kSetKind + its mask).
+constexpr int kChainKind = -1, kSetKind = 64;
 
 // Kept entries of a segment up to which they are stored one by one.
 constexpr uint32_t kFewKept = 20;
@@ -371,7 +373,8 @@ __device__ __forceinline__ void tma_scan_pass(const TmaArgs &a) {
 
 // ====================================================================== compaction
 // Fused compaction with predicate kind PK (a PredKind, or kChainKind: the
-// tests of a.chain, one after the other): CWW compute warps (tile = CWW * 512
+// tests of a.chain, one after the other; or kSetKind + a mask: those of a.set
+// at once): CWW compute warps (tile = CWW * 512
 // entries), at most MAXG blocks, NS tile slots (counts, offsets, barriers), at
 // most BMAX tiles resolved per round trip of the look-back.
 //
@@ -473,7 +476,6 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     static_assert(CWW <= 32, "the look-back warp holds one segment count per lane");
     static_assert(CWW * kSeg < 65536, "a tile aggregate fits the 16 low bits of s_pack");
     static_assert(kSeg < 65536 && RW <= 65536, "count and ring word of a segment share a word");
-    static_assert(!INTER || PK == kChainKind, "an interleaved input is compacted by a chain");
     extern __shared__ __align__(128) uint32_t stage_mem[];
     __shared__ __align__(8) uint64_t full_bar[SH], empty_bar[SH], count_bar[NS], prefix_bar[NS], mode_bar;
     __shared__ uint32_t s_wcnt[NS][CWW];  // per tile slot: segment counts (low half; above: first ring word)
@@ -738,7 +740,8 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c) v[r][c] *= mul;
             }
-            tl = tally<PK>(a.pred, v);
+            if constexpr (PK > kSetKind) tl = set_tally<PK - kSetKind>(a.set, v);
+            else tl = tally<PK>(a.pred, v);
         }
         if (vlo != 0u || vhi != uint32_t(kSeg)) tl = cut_tally(tl, vlo, vhi, lane);
         return rank_tally(tl);
@@ -759,7 +762,7 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 s_pack[k] = 0;
                 st_relaxed_u64(status_at(agg_words, tile), pack_status(epoch, kFlagAggregate, agg));
                 if (j == 0) {
-                    s_ring = agg * kRingDen <= uint32_t(T) * (PK == kChainKind ? kRingNumChain : kRingNum) ? 1u : 0u;
+                    s_ring = agg * kRingDen <= uint32_t(T) * (PK == kChainKind || PK > kSetKind ? kRingNumChain : kRingNum) ? 1u : 0u;
                     mbar_arrive(&mode_bar);
                 }
             }
@@ -1003,7 +1006,8 @@ ka_status launch_compact_shape(const TmaArgs &a, uint64_t cap, cudaStream_t stre
                                              smem, a, cap, stream);
 }
 
-// The chain's kernels of a configuration: one array, or the interleave of two.
+// The general chain's kernels of a configuration: one array, or the interleave
+// of two.
 template <int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX>
 ka_status launch_chain_config(const TmaArgs &a, uint64_t cap, cudaStream_t stream) {
     if (a.in2) return launch_compact_shape<kChainKind, CWW, SR, SH, LAG, MAXG, MINB, NS, BMAX, true>(a, cap, stream);
@@ -1011,12 +1015,12 @@ ka_status launch_chain_config(const TmaArgs &a, uint64_t cap, cudaStream_t strea
 }
 
 // One configuration's compaction for predicate kind pk (every kind has its
-// own kernel).
-template <int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX>
+// own kernel); with INTER, of the interleave of two arrays.
+template <int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX, bool INTER = false>
 ka_status launch_compact_config(const TmaArgs &a, int32_t pk, uint64_t cap, cudaStream_t stream) {
     switch (pk) {
 #define KA_CASE(K) \
-    case K: return launch_compact_shape<K, CWW, SR, SH, LAG, MAXG, MINB, NS, BMAX>(a, cap, stream);
+    case K: return launch_compact_shape<K, CWW, SR, SH, LAG, MAXG, MINB, NS, BMAX, INTER>(a, cap, stream);
         KA_CASE(kAndMaskEq0)
         KA_CASE(kLt)
         KA_CASE(kPopcOdd)
@@ -1043,6 +1047,13 @@ ka_status launch_tma_512(const TmaArgs &a, bool scan, int32_t pk, uint64_t cap, 
 ka_status launch_tma_256(const TmaArgs &a, bool scan, int32_t pk, uint64_t cap, cudaStream_t stream);
 ka_status launch_chain_768(const TmaArgs &a, uint64_t cap, cudaStream_t stream);
 ka_status launch_chain_512(const TmaArgs &a, uint64_t cap, cudaStream_t stream);
+// Shape (768, 16): one test on an interleave; a set of tests (k_tma_sets_*.cu:
+// KA_E_UNSUPPORTED for a mask of another file).
+ka_status launch_inter_768(const TmaArgs &a, int32_t pk, uint64_t cap, cudaStream_t stream);
+ka_status launch_sets_768_a(const TmaArgs &a, int mask, uint64_t cap, cudaStream_t stream);
+ka_status launch_sets_768_b(const TmaArgs &a, int mask, uint64_t cap, cudaStream_t stream);
+ka_status launch_sets_768_c(const TmaArgs &a, int mask, uint64_t cap, cudaStream_t stream);
+ka_status launch_sets_768_d(const TmaArgs &a, int mask, uint64_t cap, cudaStream_t stream);
 
 }  // namespace tma
 }  // namespace ka

@@ -3,6 +3,8 @@ and compactions, the flag/scan/move triple, and the interleave in front of
 them. Every result equals the oracle's stage-by-stage pipeline, and that of the
 same actors issued stage by stage (a failure armed far in the future on the
 first stage keeps its run apart)."""
+import itertools
+
 import numpy as np
 import pytest
 
@@ -91,6 +93,17 @@ CHAINS = {
     # five tests: a run of four, then a run of one stage
     "five": [("c", "lt", 0xF0000000, 0), ("c", "popc_odd", 0, 1), ("c", "ne", 5, 0), "map", ("c", "mod_ne0", 6, 0)],
 }
+# every set of different tests, and chains that combine or stay chains
+KINDS = {"and": ("c", "and_mask_eq0", 1, 0), "lt": ("c", "lt", 0xC0000000, 0), "popc": ("c", "popc_odd", 0, 0),
+         "mod": ("c", "mod_ne0", 6, 0), "ne": ("c", "ne", 8, 0)}
+for _r in (2, 3, 4):
+    for _c in itertools.combinations(sorted(KINDS), _r):
+        CHAINS["set " + " ".join(_c)] = [KINDS[k] for k in _c]
+CHAINS["set lt and hash"] = ["map", KINDS["lt"], ("c", "lt", 0xE0000000, 0), KINDS["and"]]
+CHAINS["one test"] = ["map", ("c", "lt", 1 << 31, 0), ("c", "lt", 1 << 30, 0)]
+CHAINS["everything"] = ["map", ("c", "lt", 0xFFFFFFFF, 0), "map"]
+CHAINS["two divisors"] = [KINDS["mod"], ("c", "mod_ne0", 5, 0)]
+CHAINS["two values"] = [KINDS["ne"], ("c", "ne", 9, 0)]
 # edges of segments, of both tile sizes (8192 and 11264 entries), of one round
 # of every resident block, and several rounds
 SIZES = [1, 3, 511, 513, 8191, 8193, 11263, 11265, 304 * 8192 + 5, (1 << 22) + 1, 152 * 11264 * 9 + 7]
