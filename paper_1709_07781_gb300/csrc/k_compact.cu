@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(BLOCK) k_compact_wave(const WaveArgs a) {
     };
     if (!a.n_ptr) load(blockIdx.x, a.n + a.lead);
     if (tid == 0) {
+        allow_dependents();
         uint32_t ep;
         bool last;
         s_ticket = take_ticket(a.ws, 0u, &ep, &last);  // one ticket per block: the last one starts the next epoch

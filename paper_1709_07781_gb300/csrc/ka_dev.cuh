@@ -291,6 +291,10 @@ __device__ __forceinline__ uint64_t *status_at(uint64_t *status, uint64_t idx) {
     return status + idx * kStatusStride;
 }
 
+// Lets a dependent launch (launch_publish) be set up from here on; it waits for
+// this kernel's end all the same. One thread per block.
+__device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Brings the sector holding *p into L2 ahead of its first use.
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 

@@ -487,6 +487,7 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     const uint32_t G = gridDim.x, b = blockIdx.x;
 
     if (tid == 0) {
+        allow_dependents();
         tma_block_setup<INTER>(a, &s_n, &s_spin, &s_epoch);
         for (int s = 0; s < SH; ++s) {
             mbar_init(&full_bar[s], 1);
