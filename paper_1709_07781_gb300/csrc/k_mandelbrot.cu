@@ -17,15 +17,16 @@
 //     exact, so this rounds as the definition's two products and a sum do
 //     (below 2^-126, where p loses bits that 2 zr zi keeps, both vanish against
 //     |ci| >= 2^-90, and for ci = 0 every term is a zero of the same sign).
-//   * The escape test runs once per four steps, on the last of them: once |z|^2 > 4 it stays so for |c|^2 <= 3.6 (|z^2 + c| >=
+//   * The escape test runs once per eight steps, on the last of them: once |z|^2 > 4 it stays so for |c|^2 <= 3.6 (|z^2 + c| >=
 //     4 - 1.898 > 2, far above the rounding), or becomes infinite or NaN, which
-//     does not compare as at most 4 either. Four steps that fail it are run
-//     again with the test on each, so the count is exact.
+//     does not compare as at most 4 either. Where eight steps fail it, the
+//     orbit at their start is kept, and looked through step by step after the
+//     loop, once for all pixels of a warp: the count is exact.
 // A pixel with |c|^2 above 3.6 (it escapes at once but for the tip at -2), or
 // with 0 < |im c| < 2^-90, goes through the definition's operations.
-// 1920 x 1080, 100 steps: 62 us with one pixel a thread and a test on every step,
-// 54 us now (35 % of the FMA pipes' issue rate, at two cycles a paired operation
-// 71 % of their time; 71 % of all issue slots).
+// 1920 x 1080, 100 steps: 63 us with one pixel a thread and a test on every step,
+// 43 us now (six paired operations a step for two pixels: 30 us at one
+// per two cycles).
 #include "ka_internal.h"
 
 namespace ka {
@@ -85,55 +86,20 @@ __device__ __forceinline__ bool paired_exact(float cr, float ci) {
     return cr * cr + ci * ci <= 3.6f && (a == 0.0f || a >= 0x1p-90f);
 }
 
-// Two orbits. A pixel that has escaped has its count in n and c = z = 0 from
-// then on, so that it never escapes again.
-struct Orbits {
-    uint64_t zr, zi, cr, ci;
-    uint32_t n[2];
-    uint32_t escaped;  // bit i: pixel i
-};
-
-// One step of both (p: zr zi), given their squares.
-__device__ __forceinline__ void advance(Orbits &o, uint64_t rr, uint64_t ii) {
-    const uint64_t p = mul_rn2(o.zr, o.zi);
-    o.zr = add_rn2(diff2(rr, ii), o.cr);
-    o.zi = fma_rn2(pair(2.0f, 2.0f), p, o.ci);
+// One step of two orbits.
+__device__ __forceinline__ void advance(uint64_t &zr, uint64_t &zi, uint64_t rr, uint64_t ii, uint64_t cr,
+                                        uint64_t ci) {
+    const uint64_t p = mul_rn2(zr, zi);
+    zr = add_rn2(diff2(rr, ii), cr);
+    zi = fma_rn2(pair(2.0f, 2.0f), p, ci);
 }
 
-// Steps k .. k + most - 1 with the test on each.
-__device__ __forceinline__ void tested_steps(Orbits &o, uint32_t k, uint32_t most) {
-#pragma unroll 1
-    for (const uint32_t end = k + most; k != end; ++k) {
-        uint64_t rr = mul_rn2(o.zr, o.zr), ii = mul_rn2(o.zi, o.zi);
-        float m[2];
-        unpair(sum2(rr, ii), m[0], m[1]);
-        if (m[0] > 4.0f || m[1] > 4.0f) {
-            float v[4][2];
-            unpair(o.zr, v[0][0], v[0][1]);
-            unpair(o.zi, v[1][0], v[1][1]);
-            unpair(o.cr, v[2][0], v[2][1]);
-            unpair(o.ci, v[3][0], v[3][1]);
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                if (m[i] > 4.0f) {
-                    o.n[i] = k;
-                    o.escaped |= 1u << i;
-                    v[0][i] = v[1][i] = v[2][i] = v[3][i] = 0.0f;
-                }
-            }
-            if (o.escaped == 3u) return;
-            o.zr = pair(v[0][0], v[0][1]);
-            o.zi = pair(v[1][0], v[1][1]);
-            o.cr = pair(v[2][0], v[2][1]);
-            o.ci = pair(v[3][0], v[3][1]);
-            rr = mul_rn2(o.zr, o.zr);
-            ii = mul_rn2(o.zi, o.zi);
-        }
-        advance(o, rr, ii);
-    }
+// a with its half i replaced by that of b.
+__device__ __forceinline__ uint64_t with_half(uint64_t a, uint64_t b, int i) {
+    return i == 0 ? (a & 0xFFFFFFFF00000000ull) | (b & 0xFFFFFFFFull) : (a & 0xFFFFFFFFull) | (b & 0xFFFFFFFF00000000ull);
 }
 
-constexpr uint32_t kMbRun = 4;  // steps between two tests
+constexpr uint32_t kMbRun = 8;  // steps between two tests
 
 __global__ void __launch_bounds__(kMbBlock) k_mandelbrot(uint32_t *out, uint32_t width, uint32_t pixels, float re_min,
                                                           float im_min, float dre, float dim, uint32_t max_iter) {
@@ -146,44 +112,76 @@ __global__ void __launch_bounds__(kMbBlock) k_mandelbrot(uint32_t *out, uint32_t
     const float ar = __fadd_rn(re_min, __fmul_rn(float(x0), dre)), ai = __fadd_rn(im_min, __fmul_rn(float(y0), dim));
     float br = __fadd_rn(re_min, __fmul_rn(float(x1), dre)), bi = __fadd_rn(im_min, __fmul_rn(float(y1), dim));
     if (!two) br = bi = 0.0f;
-    Orbits o;
-    o.n[0] = o.n[1] = max_iter;
+    uint32_t n[2] = {0u, 0u};
     if (paired_exact(ar, ai) && paired_exact(br, bi)) {
-        o.zr = o.zi = pair(0.0f, 0.0f);
-        o.cr = pair(ar, br);
-        o.ci = pair(ai, bi);
-        o.escaped = two ? 0u : 2u;
-        uint32_t k = 0u;
-        while (o.escaped != 3u && k != max_iter) {
-            uint32_t again = min(max_iter - k, kMbRun);  // steps to take with tests: a short last run, or
-            if (again == kMbRun) {
-                const Orbits start = o;
-                uint64_t norm = 0;
+        const uint64_t c0 = pair(ar, br), c1 = pair(ai, bi);
+        uint64_t zr = 0, zi = 0, cr = c0, ci = c1;  // the running orbits (a pixel that has escaped: 0, c too)
+        uint64_t sr = 0, si = 0;                    // each pixel's orbit where it is finished from, step n
+        uint32_t most[2] = {kMbRun, kMbRun};        // and the steps left to look at there
+        uint32_t escaped = two ? 0u : 2u, k = 0u;
+        for (uint32_t runs = max_iter / kMbRun; runs != 0u; --runs) {
+            const uint64_t zr_0 = zr, zi_0 = zi;
+            uint64_t norm = 0;
 #pragma unroll
-                for (uint32_t i = 0; i < kMbRun; ++i) {
-                    const uint64_t rr = mul_rn2(o.zr, o.zr), ii = mul_rn2(o.zi, o.zi);
-                    if (i == kMbRun - 1u) norm = sum2(rr, ii);
-                    advance(o, rr, ii);
-                }
-                float m[2];
-                unpair(norm, m[0], m[1]);
-                k += kMbRun;
-                if (m[0] <= 4.0f && m[1] <= 4.0f) continue;
-                k -= kMbRun;  // a run that somebody escapes in
-                o = start;
+            for (uint32_t i = 0; i < kMbRun; ++i) {
+                const uint64_t rr = mul_rn2(zr, zr), ii = mul_rn2(zi, zi);
+                if (i == kMbRun - 1u) norm = sum2(rr, ii);
+                advance(zr, zi, rr, ii, cr, ci);
             }
-            tested_steps(o, k, again);
-            k += again;
+            float m[2];
+            unpair(norm, m[0], m[1]);
+            if (!(m[0] <= 4.0f) || !(m[1] <= 4.0f)) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    if (!(m[i] <= 4.0f)) {  // in this run: found at the end, by all threads at once
+                        sr = with_half(sr, zr_0, i);
+                        si = with_half(si, zi_0, i);
+                        n[i] = k;
+                        escaped |= 1u << i;
+                        zr = with_half(zr, 0, i);
+                        zi = with_half(zi, 0, i);
+                        cr = with_half(cr, 0, i);
+                        ci = with_half(ci, 0, i);
+                    }
+                }
+                if (escaped == 3u) break;
+            }
+            k += kMbRun;
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            if (!((escaped >> i) & 1u)) {  // the last steps, fewer than a run
+                sr = with_half(sr, zr, i);
+                si = with_half(si, zi, i);
+                n[i] = k;
+                most[i] = max_iter - k;
+            }
+        }
+        uint32_t open = two ? 3u : 1u;
+#pragma unroll 1
+        for (uint32_t j = 0; j < kMbRun; ++j) {
+            const uint64_t rr = mul_rn2(sr, sr), ii = mul_rn2(si, si);
+            float m[2];
+            unpair(sum2(rr, ii), m[0], m[1]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                if (((open >> i) & 1u) && (m[i] > 4.0f || j == most[i])) {
+                    n[i] += j;
+                    open &= ~(1u << i);
+                }
+            }
+            if (open == 0u) break;
+            advance(sr, si, rr, ii, c0, c1);
         }
     } else {
-        o.n[0] = escape_steps(0.0f, 0.0f, ar, ai, max_iter);
-        if (two) o.n[1] = escape_steps(0.0f, 0.0f, br, bi, max_iter);
+        n[0] = escape_steps(0.0f, 0.0f, ar, ai, max_iter);
+        if (two) n[1] = escape_steps(0.0f, 0.0f, br, bi, max_iter);
     }
     if (two && (reinterpret_cast<uintptr_t>(out) & 7u) == 0u) {
-        *reinterpret_cast<uint2 *>(out + p0) = make_uint2(o.n[0], o.n[1]);
+        *reinterpret_cast<uint2 *>(out + p0) = make_uint2(n[0], n[1]);
     } else {
-        out[p0] = o.n[0];
-        if (two) out[p0 + 1u] = o.n[1];
+        out[p0] = n[0];
+        if (two) out[p0 + 1u] = n[1];
     }
 }
 
