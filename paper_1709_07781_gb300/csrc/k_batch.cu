@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(kBatchPlanBlock) k_batch_plan(const ka_batch_i
     __shared__ uint32_t s_warp[NW + 1];
     __shared__ uint32_t s_p, s_epoch, s_spin, s_prefix;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    wait_for_prior();
     if (tid == 0) {
         uint32_t ep;
         bool last;
@@ -280,6 +281,8 @@ __global__ void __launch_bounds__(kPlanBlock) k_gen_plan(const ka_gen_item *item
                                                           BatchLayout L, WsHeader *ws) {
     __shared__ uint64_t s_warp[33];
     __shared__ uint32_t s_tiles[kPlanBlock * kPlanIpt];
+    wait_for_prior();
+    if (threadIdx.x == 0) allow_dependents();
     uint64_t carry = 0;
     for (uint64_t base = 0; base < n_items; base += uint64_t(kPlanBlock) * kPlanIpt) {
         uint32_t nk[kPlanIpt];
@@ -335,6 +338,8 @@ constexpr int kGenBlocksPerSm = 8;
 __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSm) k_generate_batch(const ka_gen_item *items, uint32_t n_items,
                                                                const uint32_t *tile_off) {
     constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
+    wait_for_prior();
+    if (threadIdx.x == 0) allow_dependents();
     const uint32_t total = tile_off[n_items];
     if (total == 0xFFFFFFFFu) return;  // the plan kernel has recorded the error
     uint32_t t = uint32_t(uint64_t(total) * blockIdx.x / gridDim.x);
@@ -408,8 +413,8 @@ ka_status ka_compact_batch(const ka_batch_item *d_items, uint32_t n_items, uint3
     // one plan block per 256 items, each with a status word of its own
     const uint32_t plan_blocks = (n_items + kBatchPlanBlock - 1) / kBatchPlanBlock;
     if (plan_blocks > a.L.status_cap) return KA_E_WORKSPACE;
-    k_batch_plan<<<plan_blocks, kBatchPlanBlock, 0, st>>>(d_items, n_items, t.block * t.ipt, a.L, a.ws, tma, tma);
-    ka_status s = cuda_status(cudaGetLastError());
+    ka_status s = launch_dependent(k_batch_plan, plan_blocks, kBatchPlanBlock, st, d_items, n_items, t.block * t.ipt,
+                                   a.L, a.ws, tma, tma);
     if (s != KA_OK) return s;
     if (tma) return launch_batch_tma(a, t, grid, st);
     switch (shape_key(t.block, t.ipt)) {
@@ -430,12 +435,10 @@ ka_status ka_generate_batch(const ka_gen_item *d_items, uint32_t n_items, uint32
     if (n_items == 0) return KA_OK;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const BatchLayout L = batch_layout(d_ws, ws_bytes, max_items);
-    k_gen_plan<<<1, kPlanBlock, 0, st>>>(d_items, n_items, L, static_cast<WsHeader *>(d_ws));
-    ka_status s = cuda_status(cudaGetLastError());
+    ka_status s = launch_dependent(k_gen_plan, 1u, kPlanBlock, st, d_items, n_items, L, static_cast<WsHeader *>(d_ws));
     if (s != KA_OK) return s;
     const unsigned grid = unsigned(device_info().sm_count) * kGenBlocksPerSm;
-    k_generate_batch<<<grid, kGenBlock, 0, st>>>(d_items, n_items, L.tile_off);
-    return cuda_status(cudaGetLastError());
+    return launch_dependent(k_generate_batch, grid, kGenBlock, st, d_items, n_items, L.tile_off);
 }
 
 }  // extern "C"

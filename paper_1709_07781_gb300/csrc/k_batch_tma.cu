@@ -61,6 +61,7 @@ __global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_batch_tma(const BatchA
     const BatchLayout &L = a.L;
 
     if (tid == 0) {
+        allow_dependents();
         s_total = L.tile_off[a.n_items];
         const uint32_t sl = a.ws->spin_limit;
         s_spin = sl ? sl : kDefaultSpinLimit;

@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(BLOCK) k_compact_wave(const WaveArgs a) {
             v[r][3] = q.w;
         }
     };
+    wait_for_prior();
     if (!a.n_ptr) load(blockIdx.x, a.n + a.lead);
     if (tid == 0) {
         allow_dependents();
@@ -233,8 +234,7 @@ template <int BLOCK, int IPT>
 static ka_status launch_wave_shape(WaveArgs a, uint64_t cap, cudaStream_t stream) {
     const uint64_t tiles = tiles_for(cap + a.lead, BLOCK * IPT);
     if (tiles > wave_tiles<BLOCK, IPT>() || tiles > kWaveMaxTiles) return KA_E_UNSUPPORTED;
-    k_compact_wave<BLOCK, IPT><<<unsigned(tiles ? tiles : 1), BLOCK, 0, stream>>>(a);
-    return cuda_status(cudaGetLastError());
+    return launch_dependent(k_compact_wave<BLOCK, IPT>, unsigned(tiles ? tiles : 1), BLOCK, stream, a);
 }
 
 static ka_status launch_wave(const ChainLaunch &L, ka_tile t, cudaStream_t stream) {

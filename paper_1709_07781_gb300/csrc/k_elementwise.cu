@@ -195,8 +195,7 @@ ka_status launch_copy_count(const uint32_t *n_ptr, uint64_t n, uint32_t *n_out, 
 __global__ void k_publish(const uint32_t *src, uint32_t n, uint32_t fixed, const uint32_t *err, uint32_t *dst,
                           uint32_t *dst_err, uint32_t *dst_tag, uint32_t tag) {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    // (launched as a dependent: waits for the kernel before it and its stores)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_prior();
     if (!src) {
         if (t == 0) dst[0] = fixed;
     } else {
@@ -213,24 +212,11 @@ __global__ void k_publish(const uint32_t *src, uint32_t n, uint32_t fixed, const
 }
 
 ka_status launch_publish(const uint32_t *src, uint32_t n, uint32_t fixed, const uint32_t *err, uint32_t *dst,
-                         uint32_t *dst_err, cudaStream_t stream, uint32_t *dst_tag, uint32_t tag, bool dependent) {
+                         uint32_t *dst_err, cudaStream_t stream, uint32_t *dst_tag, uint32_t tag) {
     if (!dst || (err && !dst_err)) return KA_E_ARG;
     const uint32_t blocks = src && n > 256 ? std::min<uint32_t>((n + 255) / 256, 16u) : 1u;
     if (dst_tag && blocks != 1) return KA_E_ARG;
-    if (!dependent) {
-        k_publish<<<blocks, 256, 0, stream>>>(src, n, fixed, err, dst, dst_err, dst_tag, tag);
-        return cuda_status(cudaGetLastError());
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(n > 32 ? 256 : 32);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cuda_status(cudaLaunchKernelEx(&cfg, k_publish, src, n, fixed, err, dst, dst_err, dst_tag, tag));
+    return launch_dependent(k_publish, blocks, n > 32 ? 256u : 32u, stream, src, n, fixed, err, dst, dst_err, dst_tag, tag);
 }
 
 // The empty stage: one launch that does no work (prices a message-passing stage).

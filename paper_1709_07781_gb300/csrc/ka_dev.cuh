@@ -291,9 +291,12 @@ __device__ __forceinline__ uint64_t *status_at(uint64_t *status, uint64_t idx) {
     return status + idx * kStatusStride;
 }
 
-// Lets a dependent launch (launch_publish) be set up from here on; it waits for
-// this kernel's end all the same. One thread per block.
+// Dependent launches (launch_dependent). A kernel lets the next launch of the
+// stream be set up from here on (one thread per block says so); and such a
+// launch waits here until every kernel before it is complete and its stores are
+// visible.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Brings the sector holding *p into L2 ahead of its first use.
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }

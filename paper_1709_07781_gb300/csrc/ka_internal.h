@@ -90,6 +90,24 @@ inline uint32_t status_capacity(uint64_t ws_bytes) {
     return e > 0xFFFFFFFFull ? 0xFFFFFFFFu : uint32_t(e);
 }
 
+// Launches `kern` so that it may be set up while the kernel before it on the
+// stream still runs; it must wait for that kernel (wait_for_prior) before it
+// touches memory. One launch after another on a stream, 152 blocks: 3.0 us
+// plain, 1.4 us so (a cooperative launch stays at 3.1 us).
+template <class... P, class... A>
+ka_status launch_dependent(void (*kern)(P...), unsigned grid, unsigned block, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cuda_status(cudaLaunchKernelEx(&cfg, kern, P(args)...));
+}
+
 // Device ordinal and memory budget of an actor system (for the serving loop).
 ka_status system_exec_info(ka_system *sys, int *device, uint64_t *budget);
 
@@ -143,12 +161,8 @@ ka_status launch_empty(cudaStream_t stream);
 // Stores n words of src (src null: the one word `fixed`) and, if err is not
 // null, *err into host-mapped pinned memory dst / dst_err; then, if dst_tag is
 // not null (n <= 256), `tag` into dst_tag after a system-scope fence.
-// `dependent`: the launch may be set up while the kernel before it on the stream
-// still runs (the compaction kernels allow it from their start); it waits on the
-// device until that kernel is complete.
 ka_status launch_publish(const uint32_t *src, uint32_t n, uint32_t fixed, const uint32_t *err, uint32_t *dst,
-                         uint32_t *dst_err, cudaStream_t stream, uint32_t *dst_tag = nullptr, uint32_t tag = 0,
-                         bool dependent = false);
+                         uint32_t *dst_err, cudaStream_t stream, uint32_t *dst_tag = nullptr, uint32_t tag = 0);
 ka_status launch_mandelbrot(uint32_t *out, uint32_t width, uint32_t height, float re_min, float im_min, float re_max,
                             float im_max, uint32_t max_iter, uint32_t *n_out, cudaStream_t stream);
 ka_status launch_generate(uint32_t *out, uint64_t n, uint64_t seed, uint32_t *n_out, cudaStream_t stream);

@@ -870,7 +870,7 @@ static Actor *process(System *s, Actor *a, Msg *m) {
         // it knows the result is complete without asking the driver
         r->seq = r->seq + 1 ? r->seq + 1 : 1;
         pub = launch_publish(first ? first->d_count : nullptr, 1, r->pinned_count[0], err, r->pinned_dev,
-                             r->pinned_dev + 1, s->stream, r->pinned_dev + 2, r->seq, true);
+                             r->pinned_dev + 1, s->stream, r->pinned_dev + 2, r->seq);
         r->tagged = pub == KA_OK;
     }
     cudaError_t rec = cudaSuccess;
