@@ -41,22 +41,20 @@ const ka_tile kBatchOnlyShapes[] = {{704, 16}};
 
 ka_tile default_tile(int32_t kernel, uint64_t n) {
     if (kernel == KA_KERNEL_COMPACT) {
-        // Per call among others in a CUDA graph, us, 1 % / 50 % kept:
-        //   n        (256, 4)     (256, 8)     (256, 16)    (512, 16)    (768, 16)
-        //   2^12     2.7 / 3.5    2.7 / 3.4    4.0 / 4.4    6.2 / 6.9    6.7 / 7.4
-        //   2^16     4.2 / 4.2    3.4 / 3.9    4.8 / 5.0    4.4 / 4.9    6.6 / 7.0
-        //   2^18     5.2 / 5.4    3.9 / 4.0    4.3 / 5.3    4.5 / 5.1    6.7 / 6.9
-        //   2^19     6.4 / 6.1    5.7 / 5.6    4.3 / 4.8    4.3 / 4.7    6.8 / 7.1
-        //   2^20     7.7 / 7.9    6.0 / 6.3    5.4 / 5.6    4.4 / 4.8    6.6 / 6.9
-        //   2^21     12.6 / 12.9  7.5 / 8.0    8.1 / 8.3    6.5 / 7.4    6.8 / 7.2
-        //   2^23     34.8 / 37.1  21.0 / 22.7  13.0 / 14.2  10.1 / 12.4  10.9 / 11.5
-        // A register shape runs as the wave kernel while every tile of it runs
-        // at once (see k_compact.cu); the TMA shapes' set-up pays from where
-        // that kernel's status words and stores add up. (Up to 2^20 the default
-        // keeps to tiles of at most 4096 entries.)
+        // Per call among others on a stream, us, 1 % / 50 % kept:
+        //   n          (256, 8)     (512, 8)     (512, 16)    (768, 16)
+        //   200 003    4.5 / 4.5    4.6 / 4.5    8.2 / 8.2    8.3 / 8.3
+        //   524 291    5.0 / 5.3    4.9 / 5.2    6.2 / 7.2    8.2 / 8.3
+        //   1 048 576  5.7 / 6.0    5.6 / 6.0    6.2 / 7.2    8.2 / 8.2
+        //   2 400 003  8.4 / 8.6    6.7 / 7.4    9.7 / 10.3   8.3 / 8.6
+        //   4 194 309  15.8 / 16.4  14.4 / 14.9  10.3 / 10.3  10.2 / 10.3
+        // The register shapes run as the wave kernel while every tile of them
+        // runs at once (k_compact.cu): (512, 8) to 2.49 M entries, and in place
+        // of a TMA shape (512, 16) to 4.98 M. The TMA shapes are launched
+        // cooperatively, which starts about 2 us later behind another launch.
         if (n >= (1ull << 22)) return ka_tile{768, 16};
-        if (n > (1ull << 20)) return ka_tile{512, 16};
-        if (n >= 3ull << 17) return ka_tile{256, 16};
+        if (n > 2490368ull) return ka_tile{512, 16};
+        if (n >= 3ull << 17) return ka_tile{512, 8};
         return n >= (1ull << 13) ? ka_tile{256, 8} : ka_tile{256, 4};
     }
     if (kernel == KA_KERNEL_BATCH) return ka_tile{704, 16};                         // TMA batch kernel

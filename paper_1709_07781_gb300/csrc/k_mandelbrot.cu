@@ -17,9 +17,10 @@
 //     exact, so this rounds as the definition's two products and a sum do
 //     (below 2^-126, where p loses bits that 2 zr zi keeps, both vanish against
 //     |ci| >= 2^-90, and for ci = 0 every term is a zero of the same sign).
-//   * The escape test runs once per eight steps, on the last of them: once |z|^2 > 4 it stays so for |c|^2 <= 3.6 (|z^2 + c| >=
-//     4 - 1.898 > 2, far above the rounding), or becomes infinite or NaN, which
-//     does not compare as at most 4 either. Where eight steps fail it, the
+//   * The escape test runs once per eight steps, on the last of them: once
+//     |z|^2 > 4 it stays so for |c|^2 <= 3.6 (|z^2 + c| >= 4 - 1.898 > 2, far
+//     above the rounding), or becomes infinite or NaN, which does not compare as
+//     at most 4 either. Where eight steps fail it, the
 //     orbit at their start is kept, and looked through step by step after the
 //     loop, once for all pixels of a warp: the count is exact.
 // A pixel with |c|^2 above 3.6 (it escapes at once but for the tip at -2), or

@@ -122,3 +122,23 @@ def test_arrays_whose_tiles_all_run_at_once(ka, tile, off):
                 assert word(d_count) == k and ws.status(ka) == 0
                 assert np.array_equal(got[:k], y) and (got[k:] == 0xDEADBEEF).all()
         check(ka, x, tile, in_place=True)
+
+
+@pytest.mark.parametrize("n", [(3 << 17) - 1, 3 << 17, 2490367, 2490369, 3000001, 4980735, 4980737])
+@pytest.mark.parametrize("off", [0, 1])
+def test_default_kernel_by_size(ka, n, off):
+    """Calls without a shape around the sizes where the default kernel changes."""
+    x = ki.uniform_u32(n & 0xFFF, n)
+    buf = to_dev(np.concatenate([np.zeros(off, np.uint32), x]), pad=4)
+    for live in (None, n - 8191):
+        ws = Workspace(ka, n)
+        d_out, d_count = empty(n + 4), empty(1)
+        d_n = None if live is None else to_dev(np.array([live], np.uint32))
+        assert ka.ka_compact(buf.data_ptr() + 4 * off, n, d_n, ka.KA_PRED_MOD_NE0, 3, 1, d_out, d_count, ws.ptr,
+                             ws.nbytes, None, stream()) == 0
+        torch.cuda.synchronize()
+        y, k = oracle.compact(oracle.map_hash(x if live is None else x[:live]), "mod_ne0", 3)
+        got = to_host(d_out)
+        assert word(d_count) == k and ws.status(ka) == 0
+        assert np.array_equal(got[:k], y) and (got[k:] == 0xDEADBEEF).all()
+    check(ka, x, None, in_place=True)
