@@ -488,7 +488,9 @@ def actor_overhead(ka, torch):
     (N = 2^26: hash, keep top bits < 8, keep popc odd, keep % 3 != 0).
     Two direct loops: one waits with the wait the receiver uses, a completion
     tag polled in host memory, so that only the actor layer differs
-    (`overhead_pct`); the other with cudaStreamSynchronize, as plain CUDA code
+    (`overhead_pct`; in the multi-stage pipelines also that the composite's
+    stages share one kernel, which makes it far below zero: the single-stage
+    pipeline is the one that prices the layer); the other with cudaStreamSynchronize, as plain CUDA code
     would (`vs_plain_cuda_pct`). The three loops run in six interleaved
     rounds; each figure is the median round (the mean of the middle two). The
     count is even because the direct loops allocate their buffers on every

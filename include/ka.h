@@ -407,7 +407,10 @@ typedef struct ka_stage_desc {
 ka_status ka_spawn_stage(ka_system *sys, const ka_stage_desc *desc, ka_actor **out);
 /* C = B (.) A: messages to C go to A, A's result goes to B (Sec. 3.5).
  * KA_E_TYPE if A's result arity differs from B's input arity. The composite
- * holds its own references to A and B. */
+ * holds its own references to A and B. Hash maps, compactions and flag/scan/
+ * move triples that follow one another in a composite, with an interleave in
+ * front of them or not, may run as one kernel: the result, the budget and every
+ * failure are those of the stages one by one. */
 ka_status ka_compose(ka_actor *b, ka_actor *a, ka_actor **c_out);
 /* Arity of an actor's input and result messages. */
 ka_status ka_actor_arity(ka_actor *actor, int32_t *in_refs, int32_t *out_refs);
@@ -478,7 +481,8 @@ ka_status ka_bench_request_loop(ka_actor *actor, const ka_msg *msg, uint32_t ite
  * KA_BENCH_WAIT_TAG: the wait is the one ka_receive uses (a completion tag
  * that the same kernel stores last, polled in host memory; an event when the
  * length is known on the host), so the two loops differ only by the actor
- * layer. Buffers are allocated once; three untimed warm-up runs. A first
+ * layer (and, for a composite, in that its stages may share a kernel, which
+ * this loop launches one by one). Buffers are allocated once; three untimed warm-up runs. A first
  * stage KA_STAGE_PREPARE (the interleave of fuseFillsLiterals) reads its two
  * inputs from d_in: n chunk ids, then n literals. */
 #define KA_BENCH_WAIT_TAG 1u

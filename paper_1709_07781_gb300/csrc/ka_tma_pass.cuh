@@ -394,7 +394,7 @@ __device__ __forceinline__ void tma_scan_pass(const TmaArgs &a) {
 //     fifth kept it is the faster of the two (17 % kept: ring 215 us, hold
 //     220 us; 25 %: 240 us and 218 us).
 // Both are correct for any data; a block whose first tile misleads it is only
-// slower. A chain, whose tests are instructions too, holds from
+// slower. The general chain, whose switches are instructions too, holds from
 // kRingNumChain / kRingDen.
 //
 // N = 2^28, shape (768, 16), s = 1 / 5 / 10 / 25 / 50 / 99 % kept, us: 164 /
@@ -683,7 +683,7 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     // tile of an input with lead entries and in the ragged last tile, the only
     // tiles that compute the bounds (64-bit position: the last tile's later
     // segments can lie past 2^32 when T does not divide 2^32). The ragged tile
-    // is read with plain loads (zeros outside the input).
+    // is read with plain loads.
     uint32_t vlo, vhi;
     auto arrive = [&](uint32_t tile, uint32_t *seg, int s, uint32_t parity) {
         vlo = 0u;
@@ -694,17 +694,41 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
             vlo = base < a.lead ? a.lead - uint32_t(base) : 0u;
             vhi = n > base ? uint32_t(min(n - base, uint64_t(kSeg))) : 0u;
             if (!full_tile) {
+                // 16 bytes at a time, all in flight: up to 3 entries past the
+                // input's end are read, in the same 16 bytes as its last one;
+                // they and what is not read are cut from the tally
                 if constexpr (INTER) {
                     // (base is even, and so is vhi: whole pairs)
                     const uint64_t pair = base / 2;
-                    for (uint32_t e = uint32_t(lane); e < uint32_t(HALF); e += 32) {
-                        seg[e] = 2u * e < vhi ? a.in[pair + e] : 0u;
-                        seg[T / 2 + e] = 2u * e < vhi ? a.in2[pair + e] : 0u;
+                    uint4 p[2], q[2];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const uint32_t e = uint32_t(r * 128 + lane * 4);
+                        if (2u * e < vhi) {
+                            p[r] = *reinterpret_cast<const uint4 *>(a.in + pair + e);
+                            q[r] = *reinterpret_cast<const uint4 *>(a.in2 + pair + e);
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const uint32_t e = uint32_t(r * 128 + lane * 4);
+                        if (2u * e < vhi) {
+                            *reinterpret_cast<uint4 *>(seg + e) = p[r];
+                            *reinterpret_cast<uint4 *>(seg + T / 2 + e) = q[r];
+                        }
                     }
                 } else {
-                    const uint32_t *src = a.in + base;
-                    for (uint32_t e = uint32_t(lane); e < uint32_t(kSeg); e += 32)
-                        seg[e] = e >= vlo && e < vhi ? src[e] : 0u;
+                    uint4 q[ROWS];
+#pragma unroll
+                    for (int r = 0; r < ROWS; ++r) {
+                        const uint32_t e = uint32_t(r * 128 + lane * 4);
+                        if (e < vhi) q[r] = *reinterpret_cast<const uint4 *>(a.in + base + e);
+                    }
+#pragma unroll
+                    for (int r = 0; r < ROWS; ++r) {
+                        const uint32_t e = uint32_t(r * 128 + lane * 4);
+                        if (e < vhi) *reinterpret_cast<uint4 *>(seg + e) = q[r];
+                    }
                 }
                 __syncwarp();
             }
@@ -763,7 +787,7 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 s_pack[k] = 0;
                 st_relaxed_u64(status_at(agg_words, tile), pack_status(epoch, kFlagAggregate, agg));
                 if (j == 0) {
-                    s_ring = agg * kRingDen <= uint32_t(T) * (PK == kChainKind || PK > kSetKind ? kRingNumChain : kRingNum) ? 1u : 0u;
+                    s_ring = agg * kRingDen <= uint32_t(T) * (PK == kChainKind ? kRingNumChain : kRingNum) ? 1u : 0u;
                     mbar_arrive(&mode_bar);
                 }
             }
