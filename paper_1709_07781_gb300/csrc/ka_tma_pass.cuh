@@ -75,8 +75,8 @@ constexpr int kChainKind = -1, kSetKind = 64;
 // Kept entries of a segment up to which they are stored one by one.
 constexpr uint32_t kFewKept = 20;
 // Kept entries a pending tile up to which four, or two, are written out at a
-// time; and ring words kept free beyond what the last tile took.
-constexpr uint32_t kGroup4 = 64, kGroup2 = 100, kMargin = 32;
+// time.
+constexpr uint32_t kGroup4 = 64, kGroup2 = 100;
 
 // Offset of a tile's segments when its look-back gave up (no segment that
 // keeps an entry can start there: counts are at most 2^32 - 1).
@@ -391,16 +391,16 @@ __device__ __forceinline__ void tma_scan_pass(const TmaArgs &a) {
 //   * hold (more kept): SH stages; a segment is compacted in place in its
 //     stage and written out LAG tiles later, and SH - LAG stages are in
 //     flight. What bounds it is HBM (0.98-1.01 of the copy rate). Above a
-//     fifth kept it is the faster of the two (17 % kept: ring 215 us, hold
-//     220 us; 25 %: 240 us and 218 us).
+//     fifth kept it is the faster of the two (17 % kept: ring 211 us, hold
+//     220 us; 25 %: 240 us and 216 us).
 // Both are correct for any data; a block whose first tile misleads it is only
 // slower. The general chain, whose switches are instructions too, holds from
 // kRingNumChain / kRingDen.
 //
-// N = 2^28, shape (768, 16), s = 1 / 5 / 10 / 25 / 50 / 99 % kept, us: 164 /
-// 178 / 193 / 218 / 242 / 310. Before, four stages of 26 segments, each held
+// N = 2^28, shape (768, 16), s = 1 / 5 / 10 / 25 / 50 / 99 % kept, us: 163 /
+// 174 / 187 / 216 / 241 / 310. Before, four stages of 26 segments, each held
 // until its write-out unless every segment of the tile kept at most 16
-// entries: 175 / 207 / 212 / 230 / 266 / 331 (one stage in flight).
+// entries: 176 / 223 / 227 / 237 / 266 / 331 (one stage in flight).
 //
 // A segment's count is posted before its entries are stored: the other blocks
 // wait for it. A warp waits for an older tile's offset only after it has
@@ -815,7 +815,7 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
         // taken, and the next entries go to word p. A tile's entries start on
         // a 16-byte boundary.
         uint32_t *const ring = stage_mem + size_t(SR) * T + size_t(w) * RW;
-        uint32_t jq = 0, p = 0, used = 0, last = 0, s = 0, parity = 0;
+        uint32_t jq = 0, p = 0, used = 0, s = 0, parity = 0;
         auto flush = [&]() {  // the oldest tile
             const uint32_t c = s_wcnt[jq & uint32_t(NS - 1)][w], cnt = c & 0xFFFFu, off = offset(jq);
             if (off != kNoOffset) warp_ring_out<RW>(ring, c >> 16, a.out + off, cnt, lane);
@@ -851,26 +851,25 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
             used -= room;
             jq += N;
         };
+        // The oldest tiles out, of `pend` pending: several at once while they
+        // are small (the youngest of them has had three tiles' time to be
+        // resolved).
+        auto write_out = [&](uint32_t pend) {
+            if (NS >= 8 && pend >= 7u && used <= pend * kGroup4) flush_group(std::integral_constant<uint32_t, 4>{});
+            else if (NS >= 8 && pend >= 5u && used <= pend * kGroup2) flush_group(std::integral_constant<uint32_t, 2>{});
+            else flush();
+        };
         uint32_t tile = b;
         for (uint32_t j = 0; j < my_tiles; ++j, tile += G) {
-            // tile j's slot, and room for a tile that keeps a little more than
-            // the last; several tiles at once while they are small (the
-            // youngest of them has had three tiles' time to be resolved)
-            while (j - jq >= uint32_t(NS) || (jq < j && used + last + kMargin > RW)) {
-                const uint32_t pend = j - jq;
-                if (NS >= 8 && pend >= 7u && used <= pend * kGroup4) flush_group(std::integral_constant<uint32_t, 4>{});
-                else if (NS >= 8 && pend >= 5u && used <= pend * kGroup2) flush_group(std::integral_constant<uint32_t, 2>{});
-                else flush();
-            }
+            if (j - jq >= uint32_t(NS)) write_out(j - jq);  // tile j's slot
             uint32_t *const seg = seg_base + size_t(s) * T;
             if (j != 0) arrive(tile, seg, int(s), parity);
-            Ranks rk = count(seg);
+            const Ranks rk = count(seg);
             if (j != 0) post(j, tile, rk.total, p);
             const uint32_t room = (rk.total + 3u) & ~3u;
-            while (used + room > RW) {  // it keeps more than the last: make room, then count it again
-                flush();
-                rk = count(seg);
-            }
+            // room for its entries, which stay in registers meanwhile: the
+            // count is known, so nothing is written out before it has to be
+            while (used + room > RW) write_out(j - jq);
             if (rk.total <= kFewKept) {
                 // Few entries for the whole warp: each lane stores only its
                 // own kept entries, in order, reading each back from the stage
@@ -914,7 +913,6 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
             }
             p = (p + room) & (RW - 1u);
             used += room;
-            last = room;
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty_bar[s]);  // nothing of this tile is left in the stage
             if (++s == uint32_t(SR)) {
