@@ -43,11 +43,11 @@ ka_tile default_tile(int32_t kernel, uint64_t n) {
     if (kernel == KA_KERNEL_COMPACT) {
         // Per call among others on a stream, us, 1 % / 50 % kept:
         //   n          (256, 8)     (512, 8)     (512, 16)    (768, 16)
-        //   200 003    4.5 / 4.5    4.6 / 4.5    8.2 / 8.2    8.3 / 8.3
-        //   524 291    5.0 / 5.3    4.9 / 5.2    6.2 / 7.2    8.2 / 8.3
-        //   1 048 576  5.7 / 6.0    5.6 / 6.0    6.2 / 7.2    8.2 / 8.2
-        //   2 400 003  8.4 / 8.6    6.7 / 7.4    9.7 / 10.3   8.3 / 8.6
-        //   4 194 309  15.8 / 16.4  14.4 / 14.9  10.3 / 10.3  10.2 / 10.3
+        //   200 003    4.4 / 4.5    4.4 / 4.5    6.2 / 6.2    6.2 / 7.2
+        //   524 291    5.3 / 5.4    4.4 / 4.9    6.2 / 7.1    6.2 / 7.2
+        //   1 048 576  5.8 / 6.5    5.5 / 5.9    6.2 / 7.2    6.2 / 8.2
+        //   2 400 003  8.3 / 8.0    6.9 / 7.4    8.2 / 8.2    8.4 / 9.2
+        //   4 194 309  16.3 / 16.4  14.4 / 14.6  10.3 / 10.3  10.3 / 10.3
         // The register shapes run as the wave kernel while every tile of them
         // runs at once (k_compact.cu): (512, 8) to 2.49 M entries, and in place
         // of a TMA shape (512, 16) to 4.98 M. The TMA shapes are launched

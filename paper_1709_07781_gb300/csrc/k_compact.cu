@@ -312,8 +312,8 @@ ka_status launch_compact(const CompactLaunch &L, cudaStream_t stream) {
     one.chain.op[0].mul = L.mul;
     if (L.any_kernel && tma_shape(t.block, t.ipt)) {
         // tiles of 8192 entries that all run at once (4.98 M entries). Among
-        // others on a stream, 1 % / 50 % kept: 3.0 M entries 9.7 / 10.3 us on
-        // the TMA kernel, 6.6 / 8.3 us here; 4.9 M 10.3 / 10.3 and 7.5 / 8.6.
+        // others on a stream, 1 % / 50 % kept: 3.0 M entries 8.3 / 9.5 us on
+        // the TMA kernel, 6.8 / 8.2 us here; 4.9 M 10.3 / 10.3 and 7.7 / 8.8.
         const ka_status s = launch_wave(one, ka_tile{512, 16}, stream);
         if (s != KA_E_UNSUPPORTED) return s;
     }

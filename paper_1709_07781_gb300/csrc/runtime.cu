@@ -684,9 +684,9 @@ static bool actor_idle(Actor *a) {
 // pass over the run's input (launch_compact_chain), which leaves the arrays
 // between the stages unwritten: nobody but the next stage could have read
 // them. Request to response, 4-stage pipeline of N = 2^26: 267 us (four
-// kernels, 1.1 GB) became 115 us (one, 0.31 GB); interleave and zero removal
-// of 2^24 pairs: 110 us became 65 us; flag map, scan and move of 2^20 entries:
-// 41 us became 27 us.
+// kernels, 1.1 GB) became 90 us (one, 0.31 GB); interleave and zero removal of
+// 2^24 pairs: 110 us became 60 us; flag map, scan and move of 2^20 entries:
+// 41 us became 25 us.
 struct FusedRun {
     int stages = 0;  // stages of the run, from the message's (0: no run here)
     PredChain chain{};
