@@ -102,7 +102,7 @@ __device__ __forceinline__ uint64_t with_half(uint64_t a, uint64_t b, int i) {
 
 constexpr uint32_t kMbRun = 8;  // steps between two tests
 
-__global__ void __launch_bounds__(kMbBlock) k_mandelbrot(uint32_t *out, uint32_t width, uint32_t pixels, float re_min,
+__global__ void __launch_bounds__(kMbBlock, 16) k_mandelbrot(uint32_t *out, uint32_t width, uint32_t pixels, float re_min,
                                                           float im_min, float dre, float dim, uint32_t max_iter) {
     const uint64_t p0 = (uint64_t(blockIdx.x) * kMbBlock + threadIdx.x) * 2u;
     if (p0 >= pixels) return;
