@@ -332,9 +332,10 @@ __device__ __forceinline__ uint32_t splitmix64_hi(uint64_t z) {
 // an item the states of successive entries are one addition apart, and four
 // entries go out in one 16-byte store. 123 requests, 2.6e8 entries: 263 us
 // with a search and two barriers per 4096-entry tile and single-entry stores,
-// 205 us now (floor 151; what bounds it is the
+// 199 us now (floor 151; what bounds it is the
 // generator's integer work: shifts through the multiplier pipe took longer).
-constexpr int kGenBlocksPerSm = 8;
+// (blocks, groups of four in flight a thread: 8, 2: 207 us; 6, 2: 204; 6, 4: 199)
+constexpr int kGenBlocksPerSm = 6;
 __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSm) k_generate_batch(const ka_gen_item *items, uint32_t n_items,
                                                                const uint32_t *tile_off) {
     constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(kGenBlock, kGenBlocksPerSm) k_generate_batch(c
         uint64_t e = base;
         if ((reinterpret_cast<uintptr_t>(it.out) & 15u) == 0u) {  // (base is a multiple of 4)
             uint64_t z = it.seed + (base + threadIdx.x * 4u + 1u) * kGamma;
-#pragma unroll 2
+#pragma unroll 4
             for (e += threadIdx.x * 4u; e + 4u <= end; e += kGenBlock * 4u) {
                 uint4 v;
                 v.x = splitmix64_hi(z);
