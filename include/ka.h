@@ -449,6 +449,11 @@ ka_status ka_receive(ka_request_h *req, int64_t timeout_ns, ka_msg *out);
  * the library's canonicalisation, e.g. the division-free modulus test); lets
  * a CPU test compare it with the plain definition. *keep = 0 or 1. */
 ka_status ka_debug_pred_keep(int32_t pred, uint32_t param, uint32_t x, int32_t *keep);
+/* What the kernels that read 16 bytes at a time take an input of n entries at
+ * d_in for (no GPU needed): *lead entries before it in the same 16 bytes, and
+ * *first the address of the first of them; a null address and no entries when
+ * n is 0, whatever d_in is. */
+ka_status ka_debug_input_view(const uint32_t *d_in, uint64_t n, const uint32_t **first, uint32_t *lead);
 /* Test hook for the per-device launch caches (no GPU needed): looks up
  * devices[i] in order in a fresh cache whose computation for lookup i
  * returns values[i], and writes what each lookup returned to out[i]. A value

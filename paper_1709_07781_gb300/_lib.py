@@ -174,6 +174,7 @@ _SIGS = {
     "ka_receive": (ctypes.c_int32, [c_vp, ctypes.c_int64, ctypes.POINTER(ka_msg)]),
     "ka_debug_device_cache": (ctypes.c_int32, [ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32),
                                                ctypes.c_uint32, ctypes.POINTER(ctypes.c_int32)]),
+    "ka_debug_input_view": (ctypes.c_int32, [c_vp, ctypes.c_uint64, ctypes.POINTER(c_vp), c_u32p]),
     "ka_debug_pred_keep": (ctypes.c_int32, [ctypes.c_int32, ctypes.c_uint32, ctypes.c_uint32,
                                             ctypes.POINTER(ctypes.c_int32)]),
     "ka_debug_fail_stage": (ctypes.c_int32, [c_vp, ctypes.c_int32]),
@@ -389,6 +390,13 @@ def ka_debug_device_cache(devices, values):
     o = (ctypes.c_int32 * n)()
     s = lib.ka_debug_device_cache(d, v, n, o)
     return s, list(o)
+
+
+def ka_debug_input_view(d_in, n: int):
+    """(status, address of the first entry read, lead entries)."""
+    first, lead = c_vp(0), ctypes.c_uint32(0)
+    s = lib.ka_debug_input_view(ptr(d_in), n, ctypes.byref(first), ctypes.byref(lead))
+    return s, first.value or 0, lead.value
 
 
 def ka_debug_pred_keep(pred: int, param: int, x: int):

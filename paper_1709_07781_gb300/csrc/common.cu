@@ -159,6 +159,14 @@ ka_status ka_debug_pred_keep(int32_t pred, uint32_t param, uint32_t x, int32_t *
     return KA_OK;
 }
 
+ka_status ka_debug_input_view(const uint32_t *d_in, uint64_t n, const uint32_t **first, uint32_t *lead) {
+    if (!first || !lead) return KA_E_ARG;
+    const AlignedView v = aligned_view(d_in, n);
+    *first = v.in;
+    *lead = v.lead;
+    return KA_OK;
+}
+
 ka_status ka_debug_device_cache(const int32_t *devices, const int32_t *values, uint32_t n, int32_t *out) {
     if (n && (!devices || !values || !out)) return KA_E_ARG;
     PerDeviceInt cache{};

@@ -240,8 +240,9 @@ static ka_status launch_wave_shape(WaveArgs a, uint64_t cap, cudaStream_t stream
 static ka_status launch_wave(const ChainLaunch &L, ka_tile t, cudaStream_t stream) {
     if (L.n > uint64_t(kWaveMaxTiles) * t.block * t.ipt) return KA_E_UNSUPPORTED;
     WaveArgs a{};
-    a.lead = uint32_t(reinterpret_cast<uintptr_t>(L.in) & 15u) / 4u;
-    a.in = L.in - a.lead;
+    const AlignedView view = aligned_view(L.in, L.n);
+    a.lead = view.lead;
+    a.in = view.in;
     a.out = L.out;
     a.n_ptr = L.n_ptr;
     a.count = L.count;

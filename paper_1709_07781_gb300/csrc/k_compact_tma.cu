@@ -35,8 +35,9 @@ bool compact_tma_eligible(const CompactLaunch &L) {
 
 ka_status launch_compact_tma(const CompactLaunch &L, cudaStream_t stream) {
     TmaArgs a{};
-    a.lead = uint32_t(reinterpret_cast<uintptr_t>(L.in) & 15u) / 4u;
-    a.in = L.in - a.lead;
+    const AlignedView view = aligned_view(L.in, L.n);
+    a.lead = view.lead;
+    a.in = view.in;
     a.out = L.out;
     a.n_ptr = L.n_ptr;
     a.count = L.count;
@@ -121,8 +122,9 @@ ka_status launch_chain_tma(const ChainLaunch &L, ka_tile t, cudaStream_t stream)
     const ka_status ws_ok = check_workspace(L.ws, L.ws_bytes, tiles_for(entries, t.block * t.ipt));
     if (ws_ok != KA_OK) return ws_ok;
     TmaArgs a{};
-    a.lead = uint32_t(reinterpret_cast<uintptr_t>(L.in) & 15u) / 4u;
-    a.in = L.in - a.lead;
+    const AlignedView view = aligned_view(L.in, L.n);
+    a.lead = view.lead;
+    a.in = view.in;
     a.in2 = L.in2;
     a.out = L.out;
     a.n_ptr = L.n_ptr;
@@ -155,8 +157,9 @@ ka_status launch_chain_tma(const ChainLaunch &L, ka_tile t, cudaStream_t stream)
 ka_status launch_scan_tma(const uint32_t *in, uint64_t n, const uint32_t *n_ptr, uint32_t *out, uint32_t *total,
                           void *ws, uint64_t ws_bytes, ka_tile tile, cudaStream_t stream) {
     TmaArgs a{};
-    a.lead = uint32_t(reinterpret_cast<uintptr_t>(in) & 15u) / 4u;
-    a.in = in - a.lead;
+    const AlignedView view = aligned_view(in, n);
+    a.lead = view.lead;
+    a.in = view.in;
     a.out = out;
     a.out_vec = ((reinterpret_cast<uintptr_t>(out) - 4u * a.lead) & 15u) == 0 ? 1u : 0u;
     a.n_ptr = n_ptr;

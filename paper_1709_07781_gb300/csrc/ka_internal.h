@@ -108,6 +108,20 @@ ka_status launch_dependent(void (*kern)(P...), unsigned grid, unsigned block, cu
     return cuda_status(cudaLaunchKernelEx(&cfg, kern, P(args)...));
 }
 
+// The 16-byte aligned view of an input that the kernels with shifted tiles read
+// in 16-byte pieces: entry i of the input is in[lead + i], and the lead entries
+// before it lie in the same 16 bytes as its first. An input without entries has
+// none to share 16 bytes with, and its pointer may be any: its view is empty.
+struct AlignedView {
+    const uint32_t *in;
+    uint32_t lead;
+};
+inline AlignedView aligned_view(const uint32_t *in, uint64_t n) {
+    if (n == 0) return {nullptr, 0u};
+    const uint32_t lead = uint32_t(reinterpret_cast<uintptr_t>(in) & 15u) / 4u;
+    return {in - lead, lead};
+}
+
 // Device ordinal and memory budget of an actor system (for the serving loop).
 ka_status system_exec_info(ka_system *sys, int *device, uint64_t *budget);
 
