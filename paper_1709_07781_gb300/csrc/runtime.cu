@@ -725,6 +725,7 @@ static FusedRun fusable_run(const Msg *m) {
     if (st[i]->spec.kind == KA_STAGE_PREPARE) {
         const Ref *b = m->refs[1];
         if ((reinterpret_cast<uintptr_t>(x->ptr) | reinterpret_cast<uintptr_t>(b->ptr)) & 15u) return none;
+        if (!x->ptr || !b->ptr) return none;  // (the stage itself settles whether there is anything to read)
         f.inter = true;
         entries = 2 * x->capacity;
         ++i;
