@@ -390,7 +390,7 @@ ka_status launch_batch_tma_shape(const BatchArgs &a, uint32_t grid, cudaStream_t
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cuda_status(cudaLaunchKernelEx(&cfg, kern, a));
+    return launch_status(cudaLaunchKernelEx(&cfg, kern, a));
 }
 
 }  // namespace

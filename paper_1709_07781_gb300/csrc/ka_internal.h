@@ -47,6 +47,13 @@ inline ka_status launch_setup_error();
 
 // cudaError_t -> ka_status (records the CUDA error for ka_strerror detail).
 ka_status cuda_status(cudaError_t e);
+// The same for what cudaLaunchKernelEx returned: CUDA also keeps a refused
+// launch as the thread's last error, which the check after a <<<>>> launch
+// (cudaGetLastError) would report for that launch; it is taken back here.
+inline ka_status launch_status(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return cuda_status(e);
+}
 
 // Canonical device predicate for (kind, param). KA_E_ARG on an unknown kind
 // or a zero modulus.
@@ -105,7 +112,7 @@ ka_status launch_dependent(void (*kern)(P...), unsigned grid, unsigned block, cu
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cuda_status(cudaLaunchKernelEx(&cfg, kern, P(args)...));
+    return launch_status(cudaLaunchKernelEx(&cfg, kern, P(args)...));
 }
 
 // The 16-byte aligned view of an input that the kernels with shifted tiles read

@@ -1017,7 +1017,7 @@ ka_status launch_tma_kernel(Kern kern, PerDeviceInt &grid_cache, size_t smem, co
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cuda_status(cudaLaunchKernelEx(&cfg, kern, a));
+    return launch_status(cudaLaunchKernelEx(&cfg, kern, a));
 }
 
 template <int PK, int CWW, int SR, int SH, int LAG, int MAXG, int MINB, int NS, int BMAX, bool INTER = false>
