@@ -393,9 +393,19 @@ __device__ __forceinline__ void tma_scan_pass(const TmaArgs &a) {
 //     flight. What bounds it is HBM (0.98-1.01 of the copy rate). Above a
 //     fifth kept it is the faster of the two (17 % kept: ring 211 us, hold
 //     220 us; 25 %: 240 us and 216 us).
-// Both are correct for any data; a block whose first tile misleads it is only
-// slower. The general chain, whose switches are instructions too, holds from
-// kRingNumChain / kRingDen.
+// Both are correct for any data. The general chain, whose switches are
+// instructions too, holds from kRingNumChain / kRingDen.
+//
+// A block that holds goes over to rings (FOLLOW) when a tile in every lap of its
+// stages says so, at a sixteenth less than the first choice: held, data that
+// thins out waits for the look-back of every third tile. N = 2^28, 2 M entries
+// at 50 % and the rest at 0 / 1 / 2 / 5 %, us: 209 / 210 / 214 / 216 held to the
+// end, 165 / 168 / 172 / 179 so. (First tiles that keep little and a dense rest
+// stay in rings: 251 us at 50 %, where holding from the start takes 242. Following
+// the data in both directions cost every call: loops that are left and entered
+// again came out 4 to 20 % slower.) The small shapes hold to the end: following
+// cost them registers. Against a choice for every segment they lose 5 to 12 % on
+// such data, and gain 5 to 15 % on uniform data.
 //
 // N = 2^28, shape (768, 16), s = 1 / 5 / 10 / 25 / 50 / 99 % kept, us: 163 /
 // 174 / 187 / 216 / 241 / 310. Before, four stages of 26 segments, each held
@@ -415,13 +425,18 @@ constexpr uint32_t kRingNum = 3, kRingNumChain = 2, kRingDen = 16;
 
 // The producer warp's loop of a compaction block (lane 0 only): as
 // tma_produce, for SR stages or SH, whichever the compute warps choose after
-// the first tile (the first SR tiles go to the same stages either way).
-template <int SR, int SH, int T, bool INTER>
+// the first tile (the first SR tiles go to the same stages either way), or, if
+// FOLLOW, after a lap of SH stages (every stage then has had the same number of
+// tiles, so the parities are the same for all).
+template <int SR, int SH, int T, bool INTER, bool FOLLOW>
 __device__ __forceinline__ void compact_produce(const TmaArgs &a, uint32_t *stage_mem, uint64_t *full_bar,
                                                 uint64_t *empty_bar, uint64_t *mode_bar, const uint32_t *s_ring,
-                                                uint32_t my_tiles, uint32_t full_tiles) {
+                                                uint64_t *lap_bar, const uint32_t *s_leave, uint32_t my_tiles,
+                                                uint32_t full_tiles) {
     const uint32_t G = gridDim.x, b = blockIdx.x;
-    uint32_t issued = 0, stages = SR, s = 0, lap = 0;  // tile jj: stage s = jj % stages, lap = jj / stages
+    uint32_t stages = SR, s = 0, lap = 0;  // tile jj goes to stage s, which has had lap tiles before
+    uint32_t held = 0;                     // laps of SH stages
+    bool hold = false;
     for (uint32_t jj = 0; jj < my_tiles; ++jj) {
         const uint32_t tile = b + jj * G;
         if (tile >= full_tiles) break;
@@ -431,9 +446,22 @@ __device__ __forceinline__ void compact_produce(const TmaArgs &a, uint32_t *stag
                 break;
             }
             if (*s_ring == 0u) {
+                hold = true;
                 stages = SH;
                 s = SR;
                 lap = 0;
+            }
+        }
+        if (FOLLOW && hold && s == 0u) {
+            // (about as long as the wait for stage 0 would take)
+            if (!mbar_wait(lap_bar, (lap - 1u) & 1u)) {
+                record_error(a.ws, kDevErrTimeout, tile);
+                break;
+            }
+            if (*s_leave != 0u) {
+                hold = false;
+                stages = SR;
+                held = lap;
             }
         }
         if (lap != 0u && !mbar_wait(&empty_bar[s], (lap - 1u) & 1u)) {
@@ -453,15 +481,16 @@ __device__ __forceinline__ void compact_produce(const TmaArgs &a, uint32_t *stag
         const uint32_t *const h1 = INTER ? a.in2 + size_t(tile) * (T / 2) : h0 + T / 2;
         bulk_g2s(stage_mem + size_t(s) * T, h0, uint32_t(T / 2) * 4u, &full_bar[s]);
         bulk_g2s(stage_mem + size_t(s) * T + T / 2, h1, uint32_t(T / 2) * 4u, &full_bar[s]);
-        issued = jj + 1;
         if (++s == stages) {
             s = 0;
             ++lap;
         }
     }
-    // waits (bounded) for the last copies, so none lands after the block exits
-    for (uint32_t jj = issued > stages ? issued - stages : 0u; jj < issued; ++jj)
-        mbar_wait(&full_bar[jj % stages], (jj / stages) & 1u);
+    // waits (bounded) for the last copy into each stage, so none lands after the block exits
+    for (uint32_t q = 0; q < uint32_t(SH); ++q) {
+        const uint32_t tiles = q < s ? lap + 1u : q < stages ? lap : held;
+        if (tiles != 0u) mbar_wait(&full_bar[q], (tiles - 1u) & 1u);
+    }
 }
 
 template <int PK, int CWW, int SR, int SH, int LAG, int MAXG, int NS, int BMAX, bool INTER = false>
@@ -469,6 +498,8 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     constexpr int T = CWW * kSeg, ROWS = 4, HALF = kSeg / 2;
     constexpr uint32_t RW = uint32_t(SH - SR) * kSeg;  // words of a warp's ring
     constexpr int KB = (MAXG - 1 + 31) / 32;  // loads per lane for the G - 1 words before one tile
+    constexpr bool FOLLOW = SR == 3 && SH == 5;  // the shape (768, 16)
+    constexpr uint32_t RING_NUM = PK == kChainKind ? kRingNumChain : kRingNum;
     static_assert(NS >= 2 && (NS & (NS - 1)) == 0, "tile slots: a power of two");
     static_assert(SR >= 2 && SH > SR && (RW & (RW - 1)) == 0 && RW >= kSeg, "a ring: a power of two, one segment fits");
     static_assert(LAG >= 1 && LAG < SH && LAG < NS, "a held segment is written out before its stage is refilled");
@@ -482,6 +513,10 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     __shared__ uint32_t s_woff[NS][CWW];  // per tile slot: segment offsets in the output
     __shared__ uint32_t s_pack[NS];  // per tile slot: (segments counted << 16) | kept so far
     __shared__ uint32_t s_n, s_epoch, s_spin, s_ring;
+    // a block that holds: phase n - 1 of lap_bar: *s_leave says whether it goes
+    // over to the rings after lap n; left_bar: every compute warp has
+    __shared__ __align__(8) uint64_t lap_bar, left_bar;
+    __shared__ uint32_t s_leave;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t G = gridDim.x, b = blockIdx.x;
@@ -500,6 +535,11 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
         }
         mbar_init(&mode_bar, 1);
         s_ring = 0u;
+        if (FOLLOW) {
+            mbar_init(&lap_bar, 1);
+            mbar_init(&left_bar, CWW);
+            s_leave = 0u;
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -521,8 +561,8 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
 
     if (warp == CWW + 1) {
         if (lane == 0)
-            compact_produce<SR, SH, T, INTER>(a, stage_mem, full_bar, empty_bar, &mode_bar, &s_ring, my_tiles,
-                                              full_tiles);
+            compact_produce<SR, SH, T, INTER, FOLLOW>(a, stage_mem, full_bar, empty_bar, &mode_bar, &s_ring, &lap_bar,
+                                                      &s_leave, my_tiles, full_tiles);
         return;
     }
 
@@ -774,10 +814,12 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     // Posts the count of iteration j's segment, whose entries start at word p
     // of the warp's ring. The last segment counted publishes the tile aggregate
     // at once, and that of the block's first tile decides how the block uses
-    // its memory. (A warp of its own that waits for the counts and publishes
-    // takes the atomic's round trip off the compute warps, but publishes later:
-    // 241 -> 248 us at N = 2^28 and 50 % kept.)
-    auto post = [&](uint32_t j, uint32_t tile, uint32_t total, uint32_t p) {
+    // its memory (of the held tiles, one in every lap decides again, early enough
+    // for the producer, which is at most SH tiles ahead). (A warp of its own
+    // that waits for the counts and publishes takes the atomic's round trip off
+    // the compute warps, but publishes later: 241 -> 248 us at N = 2^28 and 50 %
+    // kept.)
+    auto post = [&](uint32_t j, uint32_t tile, uint32_t total, uint32_t p, auto held) {
         if (lane == 0) {
             const uint32_t k = j & uint32_t(NS - 1);
             s_wcnt[k][w] = p << 16 | total;
@@ -787,8 +829,11 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 s_pack[k] = 0;
                 st_relaxed_u64(status_at(agg_words, tile), pack_status(epoch, kFlagAggregate, agg));
                 if (j == 0) {
-                    s_ring = agg * kRingDen <= uint32_t(T) * (PK == kChainKind ? kRingNumChain : kRingNum) ? 1u : 0u;
+                    s_ring = agg * kRingDen <= uint32_t(T) * RING_NUM ? 1u : 0u;
                     mbar_arrive(&mode_bar);
+                } else if (FOLLOW && decltype(held)::value && j % uint32_t(SH) == uint32_t(SH - 3)) {
+                    s_leave = agg * kRingDen <= uint32_t(T) * (RING_NUM - 1u) ? 1u : 0u;
+                    mbar_arrive(&lap_bar);
                 }
             }
             mbar_arrive(&count_bar[k]);
@@ -806,16 +851,17 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
     };
 
     arrive(b, seg_base, 0, 0u);
-    post(0, b, count(seg_base).total, 0u);
+    post(0, b, count(seg_base).total, 0u, std::false_type{});
     if (!mbar_wait(&mode_bar, 0u) && lane == 0) record_error(a.ws, kDevErrTimeout, b);
 
-    if (s_ring != 0u) {
-        // -------------------------------------------------------------- ring
+    // -------------------------------------------------------------- ring
+    // Tiles from j0 on, from stage 0 with the parity p0 on.
+    auto ring_tiles = [&](uint32_t j0, uint32_t p0) __attribute__((always_inline)) {
         // Tile jq is the oldest one not written out; `used` ring words are
         // taken, and the next entries go to word p. A tile's entries start on
         // a 16-byte boundary.
         uint32_t *const ring = stage_mem + size_t(SR) * T + size_t(w) * RW;
-        uint32_t jq = 0, p = 0, used = 0, s = 0, parity = 0;
+        uint32_t jq = j0, p = 0, used = 0, s = 0, parity = p0;
         auto flush = [&]() {  // the oldest tile
             const uint32_t c = s_wcnt[jq & uint32_t(NS - 1)][w], cnt = c & 0xFFFFu, off = offset(jq);
             if (off != kNoOffset) warp_ring_out<RW>(ring, c >> 16, a.out + off, cnt, lane);
@@ -859,13 +905,13 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
             else if (NS >= 8 && pend >= 5u && used <= pend * kGroup2) flush_group(std::integral_constant<uint32_t, 2>{});
             else flush();
         };
-        uint32_t tile = b;
-        for (uint32_t j = 0; j < my_tiles; ++j, tile += G) {
+        uint32_t tile = b + j0 * G;
+        for (uint32_t j = j0; j < my_tiles; ++j, tile += G) {
             if (j - jq >= uint32_t(NS)) write_out(j - jq);  // tile j's slot
             uint32_t *const seg = seg_base + size_t(s) * T;
             if (j != 0) arrive(tile, seg, int(s), parity);
             const Ranks rk = count(seg);
-            if (j != 0) post(j, tile, rk.total, p);
+            if (j != 0) post(j, tile, rk.total, p, std::false_type{});
             const uint32_t room = (rk.total + 3u) & ~3u;
             // room for its entries, which stay in registers meanwhile: the
             // count is known, so nothing is written out before it has to be
@@ -921,11 +967,16 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
             }
         }
         while (jq < my_tiles) flush();
+    };
+
+    if (s_ring != 0u) {
+        ring_tiles(0u, 0u);
     } else {
         // -------------------------------------------------------------- hold
         uint32_t s = 0, parity = 0, so = 0;  // stages of tiles j and j - LAG
+        uint32_t end = my_tiles;             // the first tile that is not held
         uint32_t tile = b;
-        for (uint32_t j = 0; j < my_tiles + uint32_t(LAG); ++j, tile += G) {
+        for (uint32_t j = 0; j < end + uint32_t(LAG); ++j, tile += G) {
             if (j >= uint32_t(LAG)) {
                 const uint32_t jp = j - uint32_t(LAG), cnt = s_wcnt[jp & uint32_t(NS - 1)][w] & 0xFFFFu,
                                off = offset(jp);
@@ -942,11 +993,11 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 if (lane == 0) mbar_arrive(&empty_bar[so]);  // this warp is done with the stage
                 if (++so == uint32_t(SH)) so = 0;
             }
-            if (j < my_tiles) {
+            if (j < end) {
                 uint32_t *const seg = seg_base + size_t(s) * T;
                 if (j != 0) arrive(tile, seg, int(s), parity);
                 const Ranks rk = count(seg);
-                if (j != 0) post(j, tile, rk.total, 0u);
+                if (j != 0) post(j, tile, rk.total, 0u, std::true_type{});
                 // in place, at the front of the segment (an explicit st.shared
                 // to the segment's shared-memory address)
                 const uint32_t dst = smem_addr(seg);
@@ -972,8 +1023,20 @@ __device__ __forceinline__ void tma_compact_pass(const TmaArgs &a) {
                 if (++s == uint32_t(SH)) {
                     s = 0;
                     parity ^= 1u;
+                    if (FOLLOW && j + 1u < my_tiles) {
+                        if (!mbar_wait(&lap_bar, parity ^ 1u) && lane == 0)
+                            record_error(a.ws, kDevErrTimeout, tile);
+                        if (__any_sync(kFull, s_leave != 0u)) end = j + 1u;
+                    }
                 }
             }
+        }
+        if (FOLLOW && end != my_tiles) {
+            // Every tile before tile `end` is written out by this warp; the
+            // rings lie in stages that other warps may still be writing out of.
+            if (lane == 0) mbar_arrive(&left_bar);
+            if (!mbar_wait(&left_bar, 0u) && lane == 0) record_error(a.ws, kDevErrTimeout, b + end * G);
+            ring_tiles(end, parity);
         }
     }
 }
