@@ -111,6 +111,8 @@ Simplified simplify(const PredChain &c) {
 
 }  // namespace
 
+bool chain_is_set(const PredChain &c) { return simplify(c).mask >= 0; }
+
 // The chain kernel tests an entry with each op in turn, for any ops, at the cost
 // of a switch and a mask per op (16 entries: 20 to 30 instructions) and of two
 // to four instructions an entry; the kernels made for one test or for a set

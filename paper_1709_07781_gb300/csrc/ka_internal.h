@@ -168,6 +168,9 @@ struct ChainLaunch {
 };
 constexpr uint64_t kChainEntries = 0xFFFFFFFCull;
 ka_status launch_compact_chain(const ChainLaunch &L, cudaStream_t stream);
+// Whether the chain is one test or a set of tests (products in front of them
+// only), for which there are kernels made for it.
+bool chain_is_set(const PredChain &c);
 // The TMA kernels' chain, for the shape t or the nearest that has one.
 ka_status launch_chain_tma(const ChainLaunch &L, ka_tile t, cudaStream_t stream);
 

@@ -693,13 +693,33 @@ struct FusedRun {
     bool inter = false;  // the run starts with the interleave
 };
 
-// Appends one test to the chain; false when it is full.
-static bool chain_add(FusedRun *f, const PredDev &p, uint32_t mul) {
+// From this many entries on, a run of one array is one that kernels are made
+// for. The kernel for any chain makes every test on every entry, 1.05 us per 2^20
+// entries whatever they keep, where stages one by one stop reading what the first
+// has dropped. Three stages with a hash after the first test, which keeps 0 / 1 /
+// 10 / 50 %, one by one and as a general chain, us: 2^25 entries 47 / 58 / 71 / 97
+// and 50 / 51 / 54 / 58; 2^26 66 / 83 / 104 / 161 and 83 / 85 / 90 / 98; 2^28 173 /
+// 208 / 305 / 508 and 284 / 287 / 306 / 340. (A second phase in that kernel, for the
+// few entries that pass its first test, took longer than the tests it saved.) Runs
+// that start with the interleave gain more than that by not writing it. The
+// kernels made for a set are slower than their stages one by one only from 2^27
+// entries on and where the first test keeps next to nothing: lt, popc odd, mod 3
+// at 2^28, 0 / 0.1 / 1 / 10 %: 194 / 193 / 200 / 222 against 172 / 186 / 208 / 300.
+// (Cheap tests first, and the others on what passes them, where the warp's last
+// segment kept little: 166 / 168 / 190 / 232, and every other run 1 to 7 % longer.)
+constexpr uint64_t kSetsOnlyFrom = 1ull << 25;
+
+// Appends one test to the chain; false when it is full, or when the run would
+// no longer be one that kernels are made for, and has to be.
+static bool chain_add(FusedRun *f, const PredDev &p, uint32_t mul, bool sets_only) {
     if (f->chain.n == kChainMax) return false;
-    f->chain.op[f->chain.n].pred = p;
-    f->chain.op[f->chain.n].mul = mul;
-    f->chain.n += 1;
-    f->chain.mul_all *= mul;
+    PredChain c = f->chain;
+    c.op[c.n].pred = p;
+    c.op[c.n].mul = mul;
+    c.n += 1;
+    c.mul_all *= mul;
+    if (sets_only && !chain_is_set(c)) return false;
+    f->chain = c;
     return true;
 }
 
@@ -735,21 +755,22 @@ static FusedRun fusable_run(const Msg *m) {
     }
     if (entries > kChainEntries) return none;
     const PredDev all = {kAll, 0, 0, 0};
+    const bool sets_only = !f.inter && entries >= kSetsOnlyFrom;
     bool tests = false;
     while (i < end && usable(i)) {
         const StageSpec &sp = st[i]->spec;
         const bool shaped = sp.tile.block != 0 || sp.tile.ipt != 0;
         if (sp.kind == KA_STAGE_MAP_HASH) {
-            if (!chain_add(&f, all, kHashMul)) break;
+            if (!chain_add(&f, all, kHashMul, sets_only)) break;
             i += 1;
         } else if (sp.kind == KA_STAGE_COMPACT && !shaped) {
-            if (!chain_add(&f, sp.pred, sp.mul)) break;
+            if (!chain_add(&f, sp.pred, sp.mul, sets_only)) break;
             tests = true;
             i += 1;
         } else if (sp.kind == KA_STAGE_PREDICATE && i + 2 < end && st[i + 1]->spec.kind == KA_STAGE_EXSCAN &&
                    st[i + 2]->spec.kind == KA_STAGE_SCATTER && usable(i + 1) && usable(i + 2) &&
                    st[i + 1]->spec.tile.block == 0 && st[i + 1]->spec.tile.ipt == 0) {
-            if (!chain_add(&f, sp.pred, 1u)) break;
+            if (!chain_add(&f, sp.pred, 1u, sets_only)) break;
             tests = true;
             i += 3;
         } else {
