@@ -314,13 +314,17 @@ ka_status ka_autotune(int32_t kernel, uint64_t n, const char *cache_path, ka_til
     make_pred(KA_PRED_LT, 0x80000000u, &half);
     ka_tile win{0, 0};
     float win_us = 1e30f;
-    std::vector<ka_tile> shapes(std::begin(kShapes), std::end(kShapes));
+    // The first candidate is a call as it runs untuned: if that wins, its shape is
+    // what is kept, and calls go on as before.
+    std::vector<ka_tile> shapes(1, default_tile(kernel, n));
+    shapes.insert(shapes.end(), std::begin(kShapes), std::end(kShapes));
     shapes.insert(shapes.end(), std::begin(kTmaOnlyShapes), std::end(kTmaOnlyShapes));
     if (s == KA_OK) {
         for (const ka_tile &t : shapes) {
             auto launch = [&]() -> ka_status {
                 if (kernel == KA_KERNEL_COMPACT) {
                     CompactLaunch L{in, out, nullptr, count, n, half, 1u, ws, ws_bytes, t};
+                    L.any_kernel = &t == &shapes[0];
                     return launch_compact(L, st);
                 }
                 return launch_exclusive_scan(in, n, nullptr, out, count, ws, ws_bytes, t, st);

@@ -311,17 +311,21 @@ ka_status launch_compact(const CompactLaunch &L, cudaStream_t stream) {
     one.chain.mul_all = L.mul;
     one.chain.op[0].pred = L.pred;
     one.chain.op[0].mul = L.mul;
-    if (L.any_kernel && tma_shape(t.block, t.ipt)) {
-        // tiles of 8192 entries that all run at once (4.98 M entries). Among
-        // others on a stream, 1 % / 50 % kept: 3.0 M entries 8.3 / 9.5 us on
-        // the TMA kernel, 6.8 / 8.2 us here; 4.9 M 10.3 / 10.3 and 7.7 / 8.8.
+    if (!tma_shape(t.block, t.ipt)) {
+        const ka_status wave = launch_wave(one, t, stream);
+        if (wave != KA_E_UNSUPPORTED) return wave;
+    }
+    if (L.any_kernel) {
+        // tiles of 8192 entries that all run at once (4.98 M entries), in place
+        // of a TMA shape, or of a register shape (tuned for a smaller array of
+        // the same power of two) whose tiles do not. Among others on a stream,
+        // 1 % / 50 % kept: 3.0 M entries 8.3 / 9.5 us on the TMA kernel, 6.8 /
+        // 8.2 us here; 4.9 M 10.3 / 10.3 and 7.7 / 8.8.
         const ka_status s = launch_wave(one, ka_tile{512, 16}, stream);
         if (s != KA_E_UNSUPPORTED) return s;
     }
     if (compact_tma_eligible(L)) return launch_compact_tma(L, stream);
     if (!tile_supported(t.block, t.ipt)) return KA_E_ARG;  // a TMA-only shape beyond its size limit
-    const ka_status wave = launch_wave(one, t, stream);
-    if (wave != KA_E_UNSUPPORTED) return wave;
     CompactArgs a;
     a.in = L.in;
     a.out = L.out;
@@ -363,7 +367,7 @@ extern "C" ka_status ka_compact(const uint32_t *d_in, uint64_t n, const uint32_t
     L.ws = d_ws;
     L.ws_bytes = ws_bytes;
     L.ws_tiles = n <= 0xFFFFFFFFull ? workspace_tiles(KA_KERNEL_COMPACT, n, tile) : 0;
-    L.any_kernel = L.ws_tiles != 0;
+    L.any_kernel = !(tile && tile->block && tile->ipt);
     L.tile = resolve_tile(KA_KERNEL_COMPACT, n, tile);
     return launch_compact(L, static_cast<cudaStream_t>(stream));
 }

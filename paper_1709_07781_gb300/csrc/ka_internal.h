@@ -145,7 +145,7 @@ struct CompactLaunch {
     uint64_t ws_bytes;
     ka_tile tile;
     uint64_t ws_tiles = 0;  // tiles the workspace must hold, if more than the shape needs
-    bool any_kernel = false;  // the shape is the library's default: another kernel may run where it is faster
+    bool any_kernel = false;  // the shape is the library's choice: another kernel may run where it is faster
 };
 ka_status launch_compact(const CompactLaunch &L, cudaStream_t stream);
 // The warp-specialised TMA kernel (the TMA shapes, any 4-byte-aligned input
