@@ -132,7 +132,8 @@ bool load_table(const char *path) {
 }
 }  // namespace
 
-ka_tile resolve_tile(int32_t kernel, uint64_t n, const ka_tile *requested) {
+ka_tile resolve_tile(int32_t kernel, uint64_t n, const ka_tile *requested, uint64_t *ws_tiles) {
+    if (ws_tiles) *ws_tiles = 0;
     if (requested && requested->block && requested->ipt) return *requested;
     // The last answers of this thread, valid while the table is unchanged: a
     // pipeline stage asks the same question at every request.
@@ -141,32 +142,32 @@ ka_tile resolve_tile(int32_t kernel, uint64_t n, const ka_tile *requested) {
         int32_t kernel;
         uint64_t n;
         ka_tile tile;
+        uint64_t ws_tiles;
     };
     thread_local Memo memo[4] = {};
     thread_local uint32_t memo_next = 0;
     const uint32_t gen = g_table_gen.load(std::memory_order_acquire);
     for (const Memo &m : memo)
-        if (m.gen == gen && m.kernel == kernel && m.n == n) return m.tile;
+        if (m.gen == gen && m.kernel == kernel && m.n == n) {
+            if (ws_tiles) *ws_tiles = m.ws_tiles;
+            return m.tile;
+        }
     ka_tile t = default_tile(kernel, n);
+    uint64_t need = tiles_for(n, default_workspace_tile(kernel, n));
     {
         std::lock_guard<std::mutex> lock(g_mu);
         auto it = g_table.find({kernel, bucket_of(n)});
-        if (it != g_table.end()) t = it->second.first;
+        if (it != g_table.end()) {
+            t = it->second.first;
+            need = 0;
+        }
     }
     // The TMA kernels take at most 2^32 - 4 entries (their tiles start on a
     // 16-byte boundary); above that, a shape the register kernels also have.
     if (kernel != KA_KERNEL_BATCH && !tile_supported(t.block, t.ipt) && n > 0xFFFFFFFCull) t = ka_tile{512, 16};
-    memo[memo_next++ & 3u] = Memo{gen, kernel, n, t};  // (tagged with the generation read before the lookup)
+    memo[memo_next++ & 3u] = Memo{gen, kernel, n, t, need};  // (tagged with the generation read before the lookup)
+    if (ws_tiles) *ws_tiles = need;
     return t;
-}
-
-uint64_t workspace_tiles(int32_t kernel, uint64_t n, const ka_tile *requested) {
-    if (requested && requested->block && requested->ipt) return 0;
-    {
-        std::lock_guard<std::mutex> lock(g_mu);
-        if (g_table.count({kernel, bucket_of(n)})) return 0;
-    }
-    return tiles_for(n, default_workspace_tile(kernel, n));
 }
 
 // Times `launch` over `reps` runs after `warm` untimed runs; returns the median

@@ -366,8 +366,7 @@ extern "C" ka_status ka_compact(const uint32_t *d_in, uint64_t n, const uint32_t
     L.mul = xform == KA_XFORM_HASH ? kHashMul : 1u;
     L.ws = d_ws;
     L.ws_bytes = ws_bytes;
-    L.ws_tiles = n <= 0xFFFFFFFFull ? workspace_tiles(KA_KERNEL_COMPACT, n, tile) : 0;
     L.any_kernel = !(tile && tile->block && tile->ipt);
-    L.tile = resolve_tile(KA_KERNEL_COMPACT, n, tile);
+    L.tile = resolve_tile(KA_KERNEL_COMPACT, n, tile, &L.ws_tiles);
     return launch_compact(L, static_cast<cudaStream_t>(stream));
 }

@@ -73,12 +73,11 @@ bool batch_tma_shape(uint32_t block, uint32_t ipt);
 // Shape valid for `kernel` (a KA_KERNEL_* id).
 bool tile_supported_for(int32_t kernel, uint32_t block, uint32_t ipt);
 // Shape to use for `kernel` at size n: explicit shape, else autotuned, else default.
-ka_tile resolve_tile(int32_t kernel, uint64_t n, const ka_tile *requested);
-// Tiles that the workspace of a call must hold when it leaves the shape to the
-// library's default (0: the call or the autotuner names a shape, whose own tile
-// count is what must fit). The default shape changes with what is fastest; the
-// workspace a caller has to bring does not.
-uint64_t workspace_tiles(int32_t kernel, uint64_t n, const ka_tile *requested);
+// *ws_tiles: the tiles that the workspace of a call must hold when it leaves the
+// shape to the library's default (0: the call or the autotuner names a shape,
+// whose own tile count is what must fit). The default shape changes with what is
+// fastest; the workspace a caller has to bring does not.
+ka_tile resolve_tile(int32_t kernel, uint64_t n, const ka_tile *requested, uint64_t *ws_tiles = nullptr);
 // The batch kernel has one shape for every batch, stored under this size.
 constexpr uint64_t kBatchTileKey = 1ull << 17;
 ka_status autotune_batch(uint64_t total, const char *cache_path, ka_tile *best, float *best_us, void *stream);
