@@ -1,5 +1,5 @@
-// Compaction kernels of the TMA tile shape (768, 16) made for a set of two or
-// more tests (see k_compact_tma.cu); one of four files.
+// Compaction kernels of the TMA tile shape (768, 16) made for a set of two to
+// four tests, as many as a chain holds (see k_compact_tma.cu); one of four files.
 #include "ka_tma_pass.cuh"
 
 namespace ka {
@@ -15,7 +15,6 @@ ka_status launch_sets_768_b(const TmaArgs &a, int mask, uint64_t cap, cudaStream
         KA_CASE(19)
         KA_CASE(23)
         KA_CASE(27)
-        KA_CASE(31)
 #undef KA_CASE
     default: return KA_E_UNSUPPORTED;
     }

@@ -1,5 +1,5 @@
-// Compaction kernels of the TMA tile shape (768, 16) made for a set of two or
-// more tests (see k_compact_tma.cu); one of four files.
+// Compaction kernels of the TMA tile shape (768, 16) made for a set of two to
+// four tests, as many as a chain holds (see k_compact_tma.cu); one of four files.
 #include "ka_tma_pass.cuh"
 
 namespace ka {
