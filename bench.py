@@ -486,13 +486,13 @@ def actor_overhead(ka, torch):
     waiting for its result count on the host: the 3-actor pipeline (N = 2^20,
     keep (x & 3) == 0), its fused single-actor form, and the 4-stage pipeline
     (N = 2^26: hash, keep top bits < 8, keep popc odd, keep % 3 != 0).
-    Two direct loops: one waits with the wait the receiver uses, a completion
-    tag polled in host memory, so that only the actor layer differs
-    (`overhead_pct`; in the multi-stage pipelines also that the composite's
-    stages share one kernel, which makes it far below zero: the single-stage
-    pipeline is the one that prices the layer); the other with cudaStreamSynchronize, as plain CUDA code
-    would (`vs_plain_cuda_pct`). The three loops run in six interleaved
-    rounds; each figure is the median round (the mean of the middle two). The
+    Three direct loops: one launches the kernels that the composite launches
+    (its stages share one) and waits with the wait the receiver uses, a
+    completion tag polled in host memory, so that only the actor layer differs
+    (`overhead_pct`); one launches every stage by itself with the same wait
+    (`fusion_speedup`: its time over the first one's); and one does so and
+    waits with cudaStreamSynchronize, as plain CUDA code would
+    (`vs_plain_cuda_pct`). The four loops run in six interleaved rounds; each figure is the median round (the mean of the middle two). The
     count is even because the direct loops allocate their buffers on every
     call and run at one of two speeds, alternating from call to call (at
     2^20, 27.7 and 28.6 us per 3-actor pipeline), while the actor loop keeps
@@ -537,28 +537,34 @@ def actor_overhead(ka, torch):
             # six interleaved rounds of the three loops; medians over rounds
             n_rounds = 6
             per = max(iters // n_rounds, 1)
-            ra, rd, rt = [], [], []
+            ra, rd, rt, rs = [], [], [], []
             for _ in range(n_rounds):
                 s, t_actor, k_actor = ka.ka_bench_request_loop(pipe, msg, per, 1)
                 ka.check(s)
                 s, t_direct, k_direct = ka.ka_bench_direct_chain(specs, x, n, per)
                 ka.check(s)
-                s, t_tag, k_tag = ka.ka_bench_direct_chain(specs, x, n, per, flags=ka.KA_BENCH_WAIT_TAG)
+                s, t_tag, k_tag = ka.ka_bench_direct_chain(specs, x, n, per,
+                                                           flags=ka.KA_BENCH_WAIT_TAG | ka.KA_BENCH_SHARED)
+                ka.check(s)
+                s, t_stages, k_stages = ka.ka_bench_direct_chain(specs, x, n, per, flags=ka.KA_BENCH_WAIT_TAG)
                 ka.check(s)
                 ra.append(t_actor / per * 1e6)
                 rd.append(t_direct / per * 1e6)
                 rt.append(t_tag / per * 1e6)
-            us_a, us_d, us_t = statistics.median(ra), statistics.median(rd), statistics.median(rt)
+                rs.append(t_stages / per * 1e6)
+            us_a, us_d, us_t, us_s = (statistics.median(r) for r in (ra, rd, rt, rs))
             out.append({"pipeline": name, "n": n, "iters": n_rounds * per, "actor_us": round(us_a, 2),
                         "direct_same_wait_us": round(us_t, 2),
                         "overhead_pct": round(100.0 * (us_a / us_t - 1.0), 2),
+                        "direct_stages_us": round(us_s, 2), "fusion_speedup": round(us_s / us_t, 3),
                         "direct_plain_cuda_us": round(us_d, 2),
                         "vs_plain_cuda_pct": round(100.0 * (us_a / us_d - 1.0), 2),
                         "estimator": "median of %d interleaved rounds of %d requests" % (n_rounds, per),
                         "rounds_us": {"actor": [round(v, 2) for v in ra], "direct": [round(v, 2) for v in rd],
-                                      "direct_same_wait": [round(v, 2) for v in rt]},
+                                      "direct_same_wait": [round(v, 2) for v in rt],
+                                      "direct_stages": [round(v, 2) for v in rs]},
                         "actor_elements/s": n / (us_a * 1e-6), "count": int(k_actor),
-                        "counts_match": int(k_actor) == int(k_direct) == int(k_tag)})
+                        "counts_match": int(k_actor) == int(k_direct) == int(k_tag) == int(k_stages)})
             ka.ka_ref_release(ref)
             for a in ([pipe] if len(actors) > 1 else []) + actors:
                 ka.ka_actor_release(a)
@@ -885,20 +891,26 @@ def fuse_fills_literals_large(ka, torch, peak, k=1 << 27, zero_fraction=0.5):
                 s, pipe = ka.ka_compose(nxt, pipe)
                 ka.check(s)
             ka.check(ka.ka_bench_request_loop(pipe, msg, 3, 1)[0])
-            per, ra_us, rt_us = 10, [], []
+            per, ra_us, rt_us, rs_us = 10, [], [], []
             for _ in range(3):
                 s, t_a, k_a = ka.ka_bench_request_loop(pipe, msg, per, 1)
                 ka.check(s)
-                s, t_t, k_t = ka.ka_bench_direct_chain(specs, ab, k, per, sp, flags=ka.KA_BENCH_WAIT_TAG)
+                s, t_t, k_t = ka.ka_bench_direct_chain(specs, ab, k, per, sp,
+                                                       flags=ka.KA_BENCH_WAIT_TAG | ka.KA_BENCH_SHARED)
+                ka.check(s)
+                s, t_s, k_s = ka.ka_bench_direct_chain(specs, ab, k, per, sp, flags=ka.KA_BENCH_WAIT_TAG)
                 ka.check(s)
                 ra_us.append(t_a / per * 1e6)
                 rt_us.append(t_t / per * 1e6)
-            us_a, us_t = sorted(ra_us)[1], sorted(rt_us)[1]
+                rs_us.append(t_s / per * 1e6)
+            us_a, us_t, us_s = sorted(ra_us)[1], sorted(rt_us)[1], sorted(rs_us)[1]
             res["actor_vs_direct"].append({"pipeline": name, "actor_us": round(us_a, 1),
                                            "direct_same_wait_us": round(us_t, 1),
                                            "overhead_pct": round(100.0 * (us_a / us_t - 1.0), 2),
+                                           "direct_stages_us": round(us_s, 1),
+                                           "fusion_speedup": round(us_s / us_t, 3),
                                            "actor_pairs/s": k / (us_a * 1e-6),
-                                           "counts_match": int(k_a) == int(k_t) == kept})
+                                           "counts_match": int(k_a) == int(k_t) == int(k_s) == kept})
             for a in ([pipe] if len(actors) > 1 else []) + actors:
                 ka.ka_actor_release(a)
         ka.ka_ref_release(ra)

@@ -485,12 +485,14 @@ ka_status ka_bench_request_loop(ka_actor *actor, const ka_msg *msg, uint32_t ite
  * the wait is cudaStreamSynchronize, as plain CUDA code would wait.
  * KA_BENCH_WAIT_TAG: the wait is the one ka_receive uses (a completion tag
  * that the same kernel stores last, polled in host memory; an event when the
- * length is known on the host), so the two loops differ only by the actor
- * layer (and, for a composite, in that its stages may share a kernel, which
- * this loop launches one by one). Buffers are allocated once; three untimed warm-up runs. A first
- * stage KA_STAGE_PREPARE (the interleave of fuseFillsLiterals) reads its two
- * inputs from d_in: n chunk ids, then n literals. */
+ * length is known on the host). KA_BENCH_SHARED: stages that share a kernel when
+ * they are composed (ka_compose) share it here too; with both flags the two
+ * loops run the same kernels and differ only by the actor layer. Buffers are
+ * allocated once; three untimed warm-up runs. A first stage KA_STAGE_PREPARE
+ * (the interleave of fuseFillsLiterals) reads its two inputs from d_in: n chunk
+ * ids, then n literals. */
 #define KA_BENCH_WAIT_TAG 1u
+#define KA_BENCH_SHARED   4u
 ka_status ka_bench_direct_chain(const ka_stage_desc *stages, uint32_t n_stages, const uint32_t *d_in, uint64_t n,
                                 uint32_t iters, void *stream, uint32_t flags, double *seconds,
                                 uint64_t *last_count);

@@ -584,7 +584,7 @@ def stage_descs(specs):
     return arr
 
 
-KA_BENCH_WAIT_TAG = 1
+KA_BENCH_WAIT_TAG, KA_BENCH_SHARED = 1, 4
 
 
 def ka_bench_direct_chain(specs, d_in, n: int, iters: int, stream=None, flags: int = 0):

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "ka_internal.h"
+#include "ka_runs.h"
 
 namespace ka {
 namespace {
@@ -64,8 +65,8 @@ ka_status ka_bench_request_loop(ka_actor *actor, const ka_msg *msg, uint32_t ite
 ka_status ka_bench_direct_chain(const ka_stage_desc *stages, uint32_t n_stages, const uint32_t *d_in, uint64_t n,
                                 uint32_t iters, void *stream, uint32_t flags, double *seconds, uint64_t *last_count) {
     if (!stages || n_stages == 0 || !seconds || iters == 0 || n > 0xFFFFFFFFull) return KA_E_ARG;
-    if (flags & ~KA_BENCH_WAIT_TAG) return KA_E_ARG;
-    const bool wait_tag = (flags & KA_BENCH_WAIT_TAG) != 0;
+    if (flags & ~(KA_BENCH_WAIT_TAG | KA_BENCH_SHARED)) return KA_E_ARG;
+    const bool wait_tag = (flags & KA_BENCH_WAIT_TAG) != 0, shared = (flags & KA_BENCH_SHARED) != 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // buffers: one output (+ count word) per stage output, allocated once
     std::vector<void *> allocs;
@@ -151,16 +152,38 @@ ka_status ka_bench_direct_chain(const ka_stage_desc *stages, uint32_t n_stages, 
             *np = nullptr;
         }
     };
+    // the run that starts with stage i on the buffers c, as the actor layer plans it
+    auto run_from = [&](uint32_t i, const std::vector<Buf> &c) -> FusedRun {
+        const bool prepare = stages[i].kind == KA_STAGE_PREPARE;
+        if (c.size() != 1) return {};
+        return plan_run(
+            c[0].ptr, prepare ? c[0].ptr + c[0].cap : nullptr, c[0].cap, n_stages - i,
+            [&](size_t k) {
+                const ka_stage_desc &d = stages[i + k];
+                return RunStage{d.kind, preds[i + k], d.xform == KA_XFORM_HASH ? kHashMul : 1u,
+                                d.tile.block != 0 || d.tile.ipt != 0};
+            },
+            [](size_t) { return true; });
+    };
     auto run_once = [&]() -> ka_status {
         std::vector<Buf> c;
         c.push_back(in);
         for (uint32_t i = 0; i < n_stages; ++i) {
             const ka_stage_desc &d = stages[i];
-            const std::vector<Buf> &o = outs[i];
             uint64_t nn;
             const uint32_t *np;
             len(c[0], &nn, &np);
             ka_status e = KA_OK;
+            const FusedRun run = shared ? run_from(i, c) : FusedRun{};
+            if (run.stages) {
+                i += uint32_t(run.stages) - 1u;
+                ChainLaunch L{c[0].ptr, run.inter ? c[0].ptr + c[0].cap : nullptr, outs[i][0].ptr, np, outs[i][0].count,
+                              nn, run.chain, ws, ws_bytes};
+                if ((e = launch_compact_chain(L, st)) != KA_OK) return e;
+                c = outs[i];
+                continue;
+            }
+            const std::vector<Buf> &o = outs[i];
             switch (d.kind) {
             case KA_STAGE_MAP_HASH: e = launch_map_hash(c[0].ptr, nn, np, o[0].ptr, o[0].count, st); break;
             case KA_STAGE_COMPACT: {

@@ -37,6 +37,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "ka_internal.h"
+#include "ka_runs.h"
 
 namespace ka {
 namespace rt {
@@ -675,111 +676,27 @@ static bool actor_idle(Actor *a) {
     return !a->scheduled.load(std::memory_order_acquire) && !a->mailbox.maybe_nonempty();
 }
 
-// ---------------------------------------------------------------------------
-// Runs of stages issued as one kernel. A compaction keeps the entries that
-// pass its test, in order, so compacting a compacted array keeps the entries
-// that pass both tests; a hash map multiplies each entry; flag map, exclusive
-// scan and move together are a compaction; and the interleave only orders
-// what the compaction after it reads. A run of such stages is therefore one
-// pass over the run's input (launch_compact_chain), which leaves the arrays
-// between the stages unwritten: nobody but the next stage could have read
-// them. Request to response, 4-stage pipeline of N = 2^26: 267 us (four
-// kernels, 1.1 GB) became 90 us (one, 0.31 GB); interleave and zero removal of
-// 2^24 pairs: 110 us became 60 us; flag map, scan and move of 2^20 entries:
-// 41 us became 25 us.
-struct FusedRun {
-    int stages = 0;  // stages of the run, from the message's (0: no run here)
-    PredChain chain{};
-    bool inter = false;  // the run starts with the interleave
-};
-
-// From this many entries on, a run of one array is one that kernels are made
-// for. The kernel for any chain makes every test on every entry, 1.05 us per 2^20
-// entries whatever they keep, where stages one by one stop reading what the first
-// has dropped. Three stages with a hash after the first test, which keeps 0 / 1 /
-// 10 / 50 %, one by one and as a general chain, us: 2^25 entries 47 / 58 / 71 / 97
-// and 50 / 51 / 54 / 58; 2^26 66 / 83 / 104 / 161 and 83 / 85 / 90 / 98; 2^28 173 /
-// 208 / 305 / 508 and 284 / 287 / 306 / 340. (A second phase in that kernel, for the
-// few entries that pass its first test, took longer than the tests it saved.) Runs
-// that start with the interleave gain more than that by not writing it. The
-// kernels made for a set are slower than their stages one by one only from 2^27
-// entries on and where the first test keeps next to nothing: lt, popc odd, mod 3
-// at 2^28, 0 / 0.1 / 1 / 10 %: 194 / 193 / 200 / 222 against 172 / 186 / 208 / 300.
-// (Cheap tests first, and the others on what passes them, where the warp's last
-// segment kept little: 166 / 168 / 190 / 232, and every other run 1 to 7 % longer.)
-constexpr uint64_t kSetsOnlyFrom = 1ull << 25;
-
-// Appends one test to the chain; false when it is full, or when the run would
-// no longer be one that kernels are made for, and has to be.
-static bool chain_add(FusedRun *f, const PredDev &p, uint32_t mul, bool sets_only) {
-    if (f->chain.n == kChainMax) return false;
-    PredChain c = f->chain;
-    c.op[c.n].pred = p;
-    c.op[c.n].mul = mul;
-    c.n += 1;
-    c.mul_all *= mul;
-    if (sets_only && !chain_is_set(c)) return false;
-    f->chain = c;
-    return true;
-}
-
-// The longest run of at least two stages that starts at m's stage and holds a
-// test, as far as it can be issued as one kernel: every actor after the first
-// idle (its mail stays in order), no failure armed on any of them (each
-// counts its messages then), no tile shape asked for (the caller's choice of
-// kernel), and an input that the chain kernels take.
+// The run of stages that starts at m's stage (ka_runs.h), as far as the actors
+// allow it: every actor after the first idle (its mail stays in order), and no
+// failure armed on any of them (each counts its messages then).
 static FusedRun fusable_run(const Msg *m) {
-    FusedRun none, f;
     const std::vector<Actor *> &st = m->req->stages;
-    const size_t first = size_t(m->stage), end = st.size();
-    f.chain.mul_all = 1u;
-    auto usable = [&](size_t i) {
-        const Actor *a = st[i];
-        if (a->fail_after.load(std::memory_order_relaxed) >= 0) return false;
-        return i == first || actor_idle(st[i]);
-    };
-    if (first + 1 >= end || !usable(first) || m->n_refs != st[first]->spec.in_arity) return none;
-    size_t i = first;
-    const Ref *x = m->refs[0];
-    uint64_t entries = 0;
-    if (st[i]->spec.kind == KA_STAGE_PREPARE) {
-        const Ref *b = m->refs[1];
-        if ((reinterpret_cast<uintptr_t>(x->ptr) | reinterpret_cast<uintptr_t>(b->ptr)) & 15u) return none;
-        if (!x->ptr || !b->ptr) return none;  // (the stage itself settles whether there is anything to read)
-        f.inter = true;
-        entries = 2 * x->capacity;
-        ++i;
-    } else {
-        if (m->n_refs != 1) return none;
-        entries = x->capacity;
-    }
-    if (entries > kChainEntries) return none;
-    const PredDev all = {kAll, 0, 0, 0};
-    const bool sets_only = !f.inter && entries >= kSetsOnlyFrom;
-    bool tests = false;
-    while (i < end && usable(i)) {
-        const StageSpec &sp = st[i]->spec;
-        const bool shaped = sp.tile.block != 0 || sp.tile.ipt != 0;
-        if (sp.kind == KA_STAGE_MAP_HASH) {
-            if (!chain_add(&f, all, kHashMul, sets_only)) break;
-            i += 1;
-        } else if (sp.kind == KA_STAGE_COMPACT && !shaped) {
-            if (!chain_add(&f, sp.pred, sp.mul, sets_only)) break;
-            tests = true;
-            i += 1;
-        } else if (sp.kind == KA_STAGE_PREDICATE && i + 2 < end && st[i + 1]->spec.kind == KA_STAGE_EXSCAN &&
-                   st[i + 2]->spec.kind == KA_STAGE_SCATTER && usable(i + 1) && usable(i + 2) &&
-                   st[i + 1]->spec.tile.block == 0 && st[i + 1]->spec.tile.ipt == 0) {
-            if (!chain_add(&f, sp.pred, 1u, sets_only)) break;
-            tests = true;
-            i += 3;
-        } else {
-            break;
-        }
-    }
-    if (!tests || i - first < 2) return none;
-    f.stages = int(i - first);
-    return f;
+    const size_t first = size_t(m->stage);
+    if (first + 1 >= st.size()) return {};
+    const StageSpec &head = st[first]->spec;
+    if (m->n_refs != head.in_arity || m->n_refs != (head.kind == KA_STAGE_PREPARE ? 2 : 1)) return {};
+    const Ref *x = m->refs[0], *y = m->n_refs > 1 ? m->refs[1] : nullptr;
+    return plan_run(
+        x->ptr, y ? y->ptr : nullptr, x->capacity, st.size() - first,
+        [&](size_t i) {
+            const StageSpec &sp = st[first + i]->spec;
+            return RunStage{sp.kind, sp.pred, sp.mul, sp.tile.block != 0 || sp.tile.ipt != 0};
+        },
+        [&](size_t i) {
+            Actor *a = st[first + i];
+            if (a->fail_after.load(std::memory_order_relaxed) >= 0) return false;
+            return i == 0 || actor_idle(a);
+        });
 }
 
 // Whether the stages of a run, issued one by one, would have stayed within
