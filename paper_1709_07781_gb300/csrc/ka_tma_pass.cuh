@@ -48,7 +48,10 @@
 namespace ka {
 namespace tma {
 
-struct TmaArgs {
+// What the scan needs, and no more: with the compaction's chain and set behind it
+// as kernel parameters too, the scan of (512, 16) spilled registers and took 360
+// us at N = 2^28 instead of 334.
+struct TmaBase {
     const uint32_t *in;  // input rounded down to 16 bytes: entry i of the input is in[lead + i]
     uint32_t *out;
     const uint32_t *n_ptr;
@@ -61,6 +64,9 @@ struct TmaArgs {
     uint32_t lead;     // 0..3 entries before the input's first entry
     uint32_t out_vec;  // scan: out - lead is 16-byte aligned (output entries align with input entries)
     PredDev pred;
+};
+
+struct TmaArgs : TmaBase {
     // the chain kernels (PK == kChainKind): their tests, and for an
     // interleaved input its second array
     const uint32_t *in2;
@@ -86,7 +92,7 @@ constexpr uint32_t kNoOffset = 0xFFFFFFFFu;
 // limit and the launch epoch (one ticket per block; the last block resets).
 // With INTER, n and *n_ptr count pairs: the input has twice as many entries.
 template <bool INTER = false>
-__device__ __forceinline__ void tma_block_setup(const TmaArgs &a, uint32_t *s_n, uint32_t *s_spin,
+__device__ __forceinline__ void tma_block_setup(const TmaBase &a, uint32_t *s_n, uint32_t *s_spin,
                                                 uint32_t *s_epoch) {
     uint32_t n = a.n;
     if (a.n_ptr) {
@@ -107,7 +113,7 @@ __device__ __forceinline__ void tma_block_setup(const TmaArgs &a, uint32_t *s_n,
 // warps. Waits (bounded) for its last copies before returning, so none lands
 // after the block exits.
 template <int S, int T>
-__device__ __forceinline__ void tma_produce(const TmaArgs &a, uint32_t *stage_mem, uint64_t *full_bar,
+__device__ __forceinline__ void tma_produce(const TmaBase &a, uint32_t *stage_mem, uint64_t *full_bar,
                                             uint64_t *empty_bar, uint32_t my_tiles, uint32_t full_tiles) {
     const uint32_t G = gridDim.x, b = blockIdx.x;
     uint32_t issued = 0;
@@ -140,7 +146,7 @@ __device__ __forceinline__ void tma_produce(const TmaArgs &a, uint32_t *stage_me
 // A compute warp's segment of tile j in shared memory: waits for the copy, or
 // reads the ragged last tile with plain loads (zeros outside the input).
 // Entries [vlo, vhi) of the segment are input entries.
-__device__ __forceinline__ void tma_segment_ready(const TmaArgs &a, uint32_t *seg, uint64_t *full_bar_s,
+__device__ __forceinline__ void tma_segment_ready(const TmaBase &a, uint32_t *seg, uint64_t *full_bar_s,
                                                   uint32_t parity, bool full_tile, uint64_t base, uint32_t vlo,
                                                   uint32_t vhi, uint32_t tile, int lane) {
     if (full_tile) {
@@ -157,7 +163,7 @@ __device__ __forceinline__ void tma_segment_ready(const TmaArgs &a, uint32_t *se
 // Exclusive prefix sum: CWW compute warps (tile = CWW * 512 entries), S
 // stages, write-out LAG tiles after scanning, at most MAXG blocks.
 template <int CWW, int S, int LAG, int MAXG>
-__device__ __forceinline__ void tma_scan_pass(const TmaArgs &a) {
+__device__ __forceinline__ void tma_scan_pass(const TmaBase &a) {
     constexpr int T = CWW * kSeg, ROWS = 4;
     constexpr int K = (MAXG + 31) / 32;
     static_assert(LAG >= 1 && LAG < S && LAG <= 3, "a stage is written out before its refill; slots repeat every 4");
@@ -1047,15 +1053,15 @@ __global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_compact_tma(const TmaA
 }
 
 template <int CWW, int S, int LAG, int MAXG, int MINB>
-__global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_scan_tma(const TmaArgs a) {
+__global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_scan_tma(const TmaBase a) {
     tma_scan_pass<CWW, S, LAG, MAXG>(a);
 }
 
 // Cooperative launch of `kern` with `smem` bytes of dynamic shared memory:
 // one block per tile up to the blocks resident at once (at most MAXG),
 // found once per device.
-template <int BLOCK, int T, int MAXG, class Kern>
-ka_status launch_tma_kernel(Kern kern, PerDeviceInt &grid_cache, size_t smem, const TmaArgs &a, uint64_t cap,
+template <int BLOCK, int T, int MAXG, class Kern, class Args>
+ka_status launch_tma_kernel(Kern kern, PerDeviceInt &grid_cache, size_t smem, const Args &a, uint64_t cap,
                             cudaStream_t stream) {
     const int resident = per_device_value(grid_cache, current_device(), [&] {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
@@ -1123,8 +1129,8 @@ template <int CWW, int S, int LAG, int MAXG, int MINB>
 ka_status launch_scan_config(const TmaArgs &a, uint64_t cap, cudaStream_t stream) {
     constexpr int BLOCK = (CWW + 2) * 32, T = CWW * kSeg;
     static PerDeviceInt grid_cache;
-    return launch_tma_kernel<BLOCK, T, MAXG>(k_scan_tma<CWW, S, LAG, MAXG, MINB>, grid_cache, size_t(S) * T * 4, a,
-                                             cap, stream);
+    return launch_tma_kernel<BLOCK, T, MAXG>(k_scan_tma<CWW, S, LAG, MAXG, MINB>, grid_cache, size_t(S) * T * 4,
+                                             static_cast<const TmaBase &>(a), cap, stream);
 }
 
 // One translation unit per tile shape instantiates its configuration.
