@@ -298,47 +298,55 @@ __global__ void __launch_bounds__((CWW + 2) * 32, MINB) k_batch_tma(const BatchA
             const uint32_t base = uint32_t(w) * kSeg;
             const uint32_t vlo = ti.vlo > base ? ti.vlo - base : 0u;
             const uint32_t vhi = ti.vhi > base ? min(ti.vhi - base, uint32_t(kSeg)) : 0u;
-            uint32_t v[4][4], tl = 0;
-            if (vhi > vlo) {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint4 q = *reinterpret_cast<const uint4 *>(seg + r * 128 + lane * 4);
-                    v[r][0] = q.x;
-                    v[r][1] = q.y;
-                    v[r][2] = q.z;
-                    v[r][3] = q.w;
+            // Posted before the entries are stored: the other blocks wait for
+            // the count (and the last segment counted publishes the aggregate).
+            auto post = [&](uint32_t total) {
+                if (lane == 0) {
+                    s_wcnt[k][w] = total;
+                    const uint32_t prev = atomicAdd(&s_pack[k], (1u << 16) | total);
+                    if ((prev >> 16) == uint32_t(CWW - 1)) {
+                        s_pack[k] = 0;
+                        st_relaxed_u64(status_at(agg_words, tile),
+                                       pack_status(epoch, kFlagAggregate, (prev & 0xFFFFu) + total));
+                    }
+                    mbar_arrive(&count_bar[k]);
                 }
-                if (mul != 1u) {
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) v[r][c] *= mul;
-                }
-                // the tile's item fixes the predicate: one branch per tile into
-                // a count made for that predicate kind
-                switch (ti.pred.kind) {
-                case kAndMaskEq0: tl = tally<kAndMaskEq0>(ti.pred, v); break;
-                case kLt: tl = tally<kLt>(ti.pred, v); break;
-                case kPopcOdd: tl = tally<kPopcOdd>(ti.pred, v); break;
-                case kModNe0: tl = tally<kModNe0>(ti.pred, v); break;
-                case kNe: tl = tally<kNe>(ti.pred, v); break;
-                default: tl = tally<kAll>(ti.pred, v); break;
-                }
-                if (vlo != 0u || vhi != uint32_t(kSeg)) tl = cut_tally(tl, vlo, vhi, lane);
+            };
+            // A segment without entries, as small items have them: 20 000 items of 200
+            // entries took 171 us with these ranked too, and take 156 us.
+            if (vhi <= vlo) {
+                post(0u);
+                __syncwarp();
+                continue;
             }
+            uint32_t v[4][4], tl;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(seg + r * 128 + lane * 4);
+                v[r][0] = q.x;
+                v[r][1] = q.y;
+                v[r][2] = q.z;
+                v[r][3] = q.w;
+            }
+            if (mul != 1u) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[r][c] *= mul;
+            }
+            // the tile's item fixes the predicate: one branch per tile into
+            // a count made for that predicate kind
+            switch (ti.pred.kind) {
+            case kAndMaskEq0: tl = tally<kAndMaskEq0>(ti.pred, v); break;
+            case kLt: tl = tally<kLt>(ti.pred, v); break;
+            case kPopcOdd: tl = tally<kPopcOdd>(ti.pred, v); break;
+            case kModNe0: tl = tally<kModNe0>(ti.pred, v); break;
+            case kNe: tl = tally<kNe>(ti.pred, v); break;
+            default: tl = tally<kAll>(ti.pred, v); break;
+            }
+            if (vlo != 0u || vhi != uint32_t(kSeg)) tl = cut_tally(tl, vlo, vhi, lane);
             const Ranks rk = rank_tally(tl);
-            // posted before the entries are stored: the other blocks wait for
-            // the count (and the last segment counted publishes the aggregate)
-            if (lane == 0) {
-                s_wcnt[k][w] = rk.total;
-                const uint32_t prev = atomicAdd(&s_pack[k], (1u << 16) | rk.total);
-                if ((prev >> 16) == uint32_t(CWW - 1)) {
-                    s_pack[k] = 0;
-                    st_relaxed_u64(status_at(agg_words, tile),
-                                   pack_status(epoch, kFlagAggregate, (prev & 0xFFFFu) + rk.total));
-                }
-                mbar_arrive(&count_bar[k]);
-            }
+            post(rk.total);
             __syncwarp();  // every lane holds its entries before any is overwritten
             // in place, at the front of the segment
             const uint32_t dst = smem_addr(seg);
