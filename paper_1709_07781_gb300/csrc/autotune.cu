@@ -49,8 +49,8 @@ ka_tile default_tile(int32_t kernel, uint64_t n) {
         //   2 400 003  8.3 / 8.0    6.9 / 7.4    8.2 / 8.2    8.4 / 9.2
         //   4 194 309  16.3 / 16.4  14.4 / 14.6  10.3 / 10.3  10.3 / 10.3
         // The register shapes run as the wave kernel while every tile of them
-        // runs at once (k_compact.cu): (512, 8) to 2.49 M entries, and in place
-        // of a TMA shape (512, 16) to 4.98 M. The TMA shapes are launched
+        // runs at once (k_compact.cu): on 152 SMs (512, 8) to 2.49 M entries,
+        // and in place of another shape (512, 16) to 4.98 M. The TMA shapes are launched
         // cooperatively, which starts about 2 us later behind another launch.
         if (n >= (1ull << 22)) return ka_tile{768, 16};
         if (n > 2490368ull) return ka_tile{512, 16};

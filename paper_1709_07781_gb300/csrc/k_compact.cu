@@ -6,8 +6,9 @@
 // Output offsets never exceed input positions, so out == in is safe: a tile
 // writes only after all its predecessors have loaded their input.
 //
-// An array whose tiles all run at once (up to about 2 M entries) has a kernel of
-// its own, k_compact_wave: such a call is a chain of latencies, not of bytes.
+// An array whose tiles all run at once (up to 4.98 M entries in the largest of the
+// shapes) has a kernel of its own, k_compact_wave: such a call is a chain of
+// latencies, not of bytes.
 #include <algorithm>
 
 #include "ka_internal.h"
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(BLOCK) k_compact_fused(const CompactArgs a) {
     }
 }
 
-constexpr uint32_t kWaveMaxTiles = 1216;  // every tile reads a status word of each before it
+constexpr uint32_t kWaveMaxTiles = 1216;  // every tile reads a status word of each before it (152 SMs x 8 blocks)
 
 // One tile per block, every block running at once. What bounds it is the chain
 // ticket, loads, counts, offset, stores, a round trip to L2 or more each; so
@@ -91,6 +92,10 @@ constexpr uint32_t kWaveMaxTiles = 1216;  // every tile reads a status word of e
 //     warps' totals ranks the whole tile;
 //   * the tile starts on a 16-byte boundary of the input (up to 3 entries
 //     before it, in the same 16 bytes as its first, are read and ignored).
+// A tile whose wait gives up records the error and writes nothing. It has posted
+// its count by then, so unlike in the ticketed kernel the tiles after it are not
+// stopped: they go on with offsets that are right, and the last of them may store
+// the count. (Outputs and count are undefined once an error is recorded.)
 // A ka_compact call among others in a CUDA graph, us, at 50 % kept, against the
 // ticketed kernel below in the same shape: (256, 4), 2^16 entries 5.3 -> 4.2,
 // 2^18 6.1 -> 5.4, 2^20 9.2 -> 7.9; (512, 8), 2^18 5.4 -> 4.9, 2^20 6.4 -> 5.4,

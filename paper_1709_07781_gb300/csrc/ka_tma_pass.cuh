@@ -108,8 +108,8 @@ __device__ __forceinline__ void tma_block_setup(const TmaBase &a, uint32_t *s_n,
     *s_epoch = ep;
 }
 
-// The producer warp's loop (lane 0 only): tiles b, b + G, ... of the full
-// tiles into the S-stage ring; the ragged last tile is read by the compute
+// The producer warp's loop of a scan block (lane 0 only): tiles b, b + G, ... of
+// the full tiles into the S-stage ring; the ragged last tile is read by the compute
 // warps. Waits (bounded) for its last copies before returning, so none lands
 // after the block exits.
 template <int S, int T>
@@ -126,13 +126,11 @@ __device__ __forceinline__ void tma_produce(const TmaBase &a, uint32_t *stage_me
             break;
         }
         // the status sector of this block's tile two ahead: in L2 before its
-        // aggregate is stored and polled (first touches by those went to
-        // DRAM; 1 % faster at s = 1 %)
+        // aggregate is stored and polled
         if (jj + 2 < my_tiles) prefetch_l2(status_at(a.status, uint64_t(tile) + 2u * G));
         fence_proxy_async();  // the compute warps' accesses to this stage precede the copy into it
         mbar_expect_tx(&full_bar[s], uint32_t(T) * 4u);
-        // two copies of half a tile each, both completing on the stage's
-        // barrier (measured 0.5 % faster than one at 1 % and 50 % kept)
+        // two copies of half a tile each, both completing on the stage's barrier
         static_assert(T % 8 == 0, "each half is whole 16-byte chunks");
         bulk_g2s(stage_mem + size_t(s) * T, a.in + size_t(tile) * T, uint32_t(T / 2) * 4u, &full_bar[s]);
         bulk_g2s(stage_mem + size_t(s) * T + T / 2, a.in + size_t(tile) * T + T / 2, uint32_t(T / 2) * 4u,
@@ -143,7 +141,7 @@ __device__ __forceinline__ void tma_produce(const TmaBase &a, uint32_t *stage_me
         mbar_wait(&full_bar[jj % S], (jj / S) & 1u);
 }
 
-// A compute warp's segment of tile j in shared memory: waits for the copy, or
+// A scan warp's segment of tile j in shared memory: waits for the copy, or
 // reads the ragged last tile with plain loads (zeros outside the input).
 // Entries [vlo, vhi) of the segment are input entries.
 __device__ __forceinline__ void tma_segment_ready(const TmaBase &a, uint32_t *seg, uint64_t *full_bar_s,
