@@ -10,6 +10,7 @@ pytestmark = pytest.mark.gpu
 
 import ka_inputs as ki  # noqa: E402
 import oracle  # noqa: E402
+from gpu_util import Workspace, empty, stream, to_dev, to_host, word  # noqa: E402
 from test_gpu_compact_modes import HALF, check, ka, with_density  # noqa: E402,F401
 from test_gpu_fused_runs import expected, request, spawn_all, system  # noqa: E402,F401
 from test_gpu_actors import compose  # noqa: E402
@@ -42,6 +43,29 @@ def test_patterns(ka, pattern):  # noqa: F811
     x = with_density(d.size, d, 17)
     check(ka, x, TILE)
     check(ka, x, TILE, in_place=True)
+
+
+def test_a_look_back_that_gives_up(ka):  # noqa: F811
+    """One poll, then no more: blocks whose look-back gives up still count, change
+    over and end; the next call in the same workspace, cleared, is right."""
+    d = by_round([0.8] * 4 + [0.01] * 12, 9)
+    x = with_density(d.size, d, 41)
+    ws = Workspace(ka, x.size, TILE)
+    d_x, d_out, d_count = to_dev(x, pad=4), empty(x.size + 4), empty(1)
+
+    def call():
+        assert ka.ka_compact(d_x, x.size, None, ka.KA_PRED_LT, HALF, 0, d_out, d_count, ws.ptr, ws.nbytes, TILE,
+                             stream()) == 0
+        torch.cuda.synchronize()
+        return ws.status(ka)
+
+    assert ka.ka_workspace_set_spin_limit(ws.ptr, 1, stream()) == 0
+    for _ in range(3):
+        assert call() in (0, ka.KA_E_DEVICE_TIMEOUT)
+    assert ka.ka_workspace_init(ws.ptr, ws.nbytes, stream()) == 0
+    assert call() == 0
+    y, k = oracle.compact(x, "lt", HALF)
+    assert word(d_count) == k and np.array_equal(to_host(d_out, k), y)
 
 
 RUNS = {
